@@ -509,6 +509,9 @@ cudaError_t launch_bin(const BinArgs &a, cudaStream_t s);
 // Stable LSD radix sort of (key, value) pairs on bits [0, bits), 8 bits a pass (binning.cu).
 cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], bool iota_vals, const uint32_t *n_dev,
                        uint32_t n_host_max, int bits, uint32_t *hist, uint32_t *partials, cudaStream_t s);
+// Exclusive scan of n uint32 (binning.cu); partials: ceil(n / kScanTile) + 1 words. In place is allowed.
+cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *partials, uint32_t *total,
+                           cudaStream_t s);
 cudaError_t launch_render_fwd(const FwdArgs &a, cudaStream_t s);
 cudaError_t launch_render_bwd(const BwdArgs &a, cudaStream_t s);
 bool tile_shape_supported(int tw, int th);

@@ -2,19 +2,18 @@
 // the 16 splats closest to the splat it was drawn from).
 //
 // A uniform grid over the centres' bounding box, at most two cells per point, is
-// built on the device: cell keys, a stable radix sort of the points by cell (the
-// sort of the binning), dense cell ranges and a cell-ordered copy of the centres.
-// Each query then walks Chebyshev rings of cells around its own cell, keeping its 16
-// best (distance, index) pairs sorted in registers, and stops once the 16th best
-// distance is within the distance from the query to the part of the grid's box outside
-// the searched block (no unsearched point can be closer). Once it holds 16, rows and
-// cells whose box lies farther than the 16th are skipped without reading their ranges,
-// which keeps queries away from the centres (points in front of a surface) from reading
-// every cell of their block. Queries run in cell order, so a warp searches one
+// built on the device: cell keys and counts, a stable radix sort of the points by cell (the
+// sort of the binning), the scan of the counts (the first centre of every cell, so that a run of
+// cells along x is one range of centres, read with two loads) and a cell-ordered copy of the centres.
+// A query walks Chebyshev rings of cells around its own cell twice: first for the 16 least
+// distances alone, then, over the cells within the 16th, for the centres themselves. Rows of
+// cells farther than the current 16th are skipped and the others cut to it along x, which keeps
+// queries away from the centres (points in front of a surface) from reading every cell of their
+// block. Queries run in cell order, so a warp searches one
 // neighbourhood. Distances are squared float32 with a fixed operation order; ties go to
-// the lower index. A query examines at most 65,536 candidates (a bound that well-spread
-// centres never reach; tens of thousands of coincident centres would), so no input makes
-// the search quadratic.
+// the lower index. A query that would examine more than 65,536 candidates (a bound that well-spread
+// centres never reach; tens of thousands of coincident centres would) takes the best of the first
+// 65,536 in ring order instead, so no input makes the search quadratic.
 #include "ges_internal.cuh"
 
 namespace ges {
@@ -23,6 +22,13 @@ namespace {
 
 constexpr int kK = GES_KNN_K;
 constexpr uint32_t kQueryBudget = 1u << 16;  // candidate points one query may examine
+// 16 CTAs of 64 threads per SM (64 registers): at 12 or 20 the centre queries take 11 % or 1 % longer
+constexpr int kQueryThreads = 64, kQueryCtas = 16;
+// The first pass ends when the searched cells reach sqrt(kReach) of the 16th distance: the second pass then
+// drops the few candidates too many, which costs less than another ring (reach 1: 1.61 ms against 1.42-1.45
+// at 0.25 and 0.5 for the centres; level-set queries 3.93 against 3.78 ms).
+constexpr float kReach = 0.25f;
+constexpr int kNearRings = 4;  // rings of cells that a point query tries before it walks blocks
 
 struct KnnGrid {
     float lo[3];
@@ -32,7 +38,7 @@ struct KnnGrid {
 };
 
 struct KnnLayout {
-    uint64_t bbox, grid, keys0, keys1, vals0, vals1, hist, partials, ranges, bcount, spos, bytes;
+    uint64_t bbox, grid, keys0, keys1, vals0, vals1, hist, partials, starts, bcount, spos, bytes;
     uint32_t cap_cells, nblocks;
     int bits;
 };
@@ -43,7 +49,7 @@ KnnLayout knn_layout(int32_t n) {
     KnnLayout L;
     uint64_t cap = 2ull * (uint64_t)n;
     if (cap < 1) cap = 1;
-    if (cap > (1ull << 27)) cap = 1ull << 27;
+    if (cap > (1ull << 26) - 1) cap = (1ull << 26) - 1;  // one scan covers the cells and the end
     L.cap_cells = (uint32_t)cap;
     L.bits = 1;
     while ((1ull << L.bits) < cap) ++L.bits;
@@ -56,8 +62,9 @@ KnnLayout knn_layout(int32_t n) {
     L.vals0 = off; off = al256(off + 4ull * n);
     L.vals1 = off; off = al256(off + 4ull * n);
     L.hist = off; off = al256(off + 4ull * 256 * L.nblocks);
-    L.partials = off; off = al256(off + 4ull * (ceil_div_u64(256ull * L.nblocks, kScanTile) + 1));
-    L.ranges = off; off = al256(off + 8ull * L.cap_cells);
+    const uint64_t scanned = 256ull * L.nblocks > cap + 1 ? 256ull * L.nblocks : cap + 1;
+    L.partials = off; off = al256(off + 4ull * (ceil_div_u64(scanned, kScanTile) + 1));
+    L.starts = off; off = al256(off + 4ull * (L.cap_cells + 1ull));
     L.bcount = off; off = al256(off + 4ull * L.cap_cells);  // blocks <= cells <= cap_cells
     L.spos = off; off = al256(off + 16ull * n);
     L.bytes = off;
@@ -147,7 +154,7 @@ __device__ __forceinline__ int cell_axis(float p, float lo, float inv_h, int dim
 __device__ __forceinline__ int block_dim(int d) { return (d + 1) >> 1; }
 
 __global__ void __launch_bounds__(256) k_knn_keys(const float4 *pos, int n, const KnnGrid *g, uint32_t *keys,
-                                                  uint32_t *bcount) {
+                                                  uint32_t *ccount, uint32_t *bcount) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float4 p = __ldg(pos + i);
@@ -155,20 +162,25 @@ __global__ void __launch_bounds__(256) k_knn_keys(const float4 *pos, int n, cons
     const int cx = cell_axis(p.x, G.lo[0], G.inv_h, G.dims[0]);
     const int cy = cell_axis(p.y, G.lo[1], G.inv_h, G.dims[1]);
     const int cz = cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2]);
-    keys[i] = (uint32_t)(cx + G.dims[0] * (cy + G.dims[1] * cz));
+    const uint32_t cell = (uint32_t)(cx + G.dims[0] * (cy + G.dims[1] * cz));
+    keys[i] = cell;
+    atomicAdd(ccount + cell, 1u);
     atomicAdd(bcount + ((cx >> 1) + block_dim(G.dims[0]) * ((cy >> 1) + block_dim(G.dims[1]) * (cz >> 1))), 1u);
 }
 
-__global__ void __launch_bounds__(256) k_knn_ranges(const uint32_t *keys, const uint32_t *idx, const float4 *pos,
-                                                    int n, uint2 *ranges, float4 *spos) {
+// The centres in cell order.
+__global__ void __launch_bounds__(256) k_knn_gather(const uint32_t *idx, const float4 *pos, int n, float4 *spos) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const uint32_t k = keys[r];
-    if (r == 0 || keys[r - 1] != k) ranges[k].x = (uint32_t)r;
-    if (r == n - 1 || keys[r + 1] != k) ranges[k].y = (uint32_t)r + 1;
     const uint32_t i = idx[r];
     const float4 p = __ldg(pos + i);
     spos[r] = make_float4(p.x, p.y, p.z, __uint_as_float(i));
+}
+
+// The centres of cells [first, last] of one row, consecutive in cell order (none if first > last).
+__device__ __forceinline__ uint2 row_range(const uint32_t *starts, int first, int last) {
+    if (first > last) return make_uint2(0u, 0u);
+    return make_uint2(__ldg(starts + first), __ldg(starts + last + 1));
 }
 
 __device__ __forceinline__ float dist2(float4 a, float4 b) {
@@ -201,7 +213,7 @@ __device__ __forceinline__ void scan_cell(float4 p, uint2 rg, const float4 *spos
 }
 
 // Ring search around point p for its kK nearest centres (lists in bd / bi, sorted).
-__device__ __forceinline__ void ring_search(float4 p, const KnnGrid &G, const uint2 *ranges, const float4 *spos,
+__device__ __forceinline__ void ring_search(float4 p, const KnnGrid &G, const uint32_t *starts, const float4 *spos,
                                             float (&bd)[kK], uint32_t (&bi)[kK]) {
     const int c[3] = {cell_axis(p.x, G.lo[0], G.inv_h, G.dims[0]), cell_axis(p.y, G.lo[1], G.inv_h, G.dims[1]),
                       cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2])};
@@ -230,7 +242,8 @@ __device__ __forceinline__ void ring_search(float4 p, const KnnGrid &G, const ui
         auto visit = [&](int cx, int cy, int cz, float gyz) {
             const float gx = gap(0, cx);
             if (fmaf(gx, gx, gyz) > bd[kK - 1]) return;
-            scan_cell(p, __ldg(ranges + (cx + G.dims[0] * (cy + G.dims[1] * cz))), spos, examined, bd, bi);
+            const int cell = cx + G.dims[0] * (cy + G.dims[1] * cz);
+            scan_cell(p, row_range(starts, cell, cell), spos, examined, bd, bi);
         };
         // the cells at Chebyshev distance `ring` from the query's cell
         for (int cz = z0; cz <= z1; ++cz) {
@@ -281,7 +294,7 @@ __device__ __forceinline__ float slab_gap(float lo, float w, float slack, float 
 // space (start points in front of a surface, rays past its edge): a block whose box lies
 // farther than the 16th candidate, or that holds no centre, costs one test and at most one
 // count read; the cells of the others are pruned and scanned as in ring_search.
-__device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const uint2 *ranges, const uint32_t *bcount,
+__device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const uint32_t *starts, const uint32_t *bcount,
                                              const float4 *spos, float (&bd)[kK], uint32_t (&bi)[kK]) {
     const int dx = G.dims[0], dy = G.dims[1], dz = G.dims[2];
     const int bx_n = block_dim(dx), by_n = block_dim(dy), bz_n = block_dim(dz);
@@ -315,7 +328,8 @@ __device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const ui
                     for (int fx = 2 * bx; fx <= fx1; ++fx) {
                         const float hx = slab_gap(lx, h, sl, p.x, fx);
                         if (fmaf(hx, hx, hyz) > bd[kK - 1]) continue;
-                        scan_cell(p, __ldg(ranges + (fx + dx * (fy + dy * fz))), spos, examined, bd, bi);
+                        const int cell = fx + dx * (fy + dy * fz);
+                        scan_cell(p, row_range(starts, cell, cell), spos, examined, bd, bi);
                     }
                 }
             }
@@ -355,17 +369,225 @@ __device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const ui
     }
 }
 
-__global__ void __launch_bounds__(128) k_knn_query(const float4 *spos, const uint2 *ranges, const KnnGrid *gp, int n,
-                                                   int32_t *knn) {
+// ---------------------------------------------------------------------------
+// Two-pass search, one thread per query. It is bound by instruction issue under divergence (14 of 32 lanes
+// active: the lanes' ranges of centres differ in length). Keeping 16 (distance, index) pairs sorted while scanning costs
+// about seven instructions a slot for every candidate that any lane of the warp accepts, which is nearly
+// all of them. The first pass keeps the 16 least distances alone (a minimum and a maximum a slot) and ends
+// with a distance that at least 16 centres lie within; the second walks the cells within it and appends
+// the candidates to the thread's column of a shared table, which is sorted once at the end.
+// 1.5M centres of a heightfield, the whole call: 2.61 ms with one pass of pair insertion -> 1.82 (two passes,
+// 64 registers) -> 1.44 (rows cut to the bound, middle rows first) -> 1.26 ms (scanned cell counts in
+// place of a range per cell). A warp per query (candidates across the lanes, a warp-wide sort) was
+// exact too but took 3.2 ms.
+
+// Inserts d into the sorted bd[0..kK) (a NaN or a distance beyond the last leaves it unchanged).
+__device__ __forceinline__ void insert_dist(float d, float (&bd)[kK]) {
+    if (!(d < bd[kK - 1])) return;
+#pragma unroll
+    for (int k = kK - 1; k > 0; --k) bd[k] = fminf(bd[k], fmaxf(bd[k - 1], d));
+    bd[0] = fminf(bd[0], d);
+}
+
+// A thread's table column: up to kK candidates (distance, index), unsorted, `stride` apart.
+struct Found {
+    uint2 *col;
+    int stride, n;
+};
+
+// Adds (d, id); a full column replaces its greatest pair if (d, id) comes before it.
+__device__ __forceinline__ void add_found(Found &f, float d, uint32_t id) {
+    const uint32_t db = __float_as_uint(d);  // d >= 0: bit patterns order as the values do
+    if (f.n < kK) {
+        f.col[f.n * f.stride] = make_uint2(db, id);
+        ++f.n;
+        return;
+    }
+    int worst = 0;
+    uint2 w = f.col[0];
+    for (int k = 1; k < kK; ++k) {
+        const uint2 c = f.col[k * f.stride];
+        if (c.x > w.x || (c.x == w.x && c.y > w.y)) { w = c; worst = k; }
+    }
+    if (db < w.x || (db == w.x && id < w.y)) f.col[worst * f.stride] = make_uint2(db, id);
+}
+
+// The column sorted by (distance, index), as indices; missing entries -1. Batcher's odd-even merge sort.
+__device__ __forceinline__ void sorted_indices(const Found &f, int32_t (&out)[kK]) {
+    unsigned long long key[kK];
+#pragma unroll
+    for (int k = 0; k < kK; ++k) {
+        const uint2 c = f.col[k * f.stride];
+        key[k] = k < f.n ? ((unsigned long long)c.x << 32) | c.y : ~0ull;
+    }
+#pragma unroll
+    for (int p = 1; p < kK; p <<= 1)
+#pragma unroll
+        for (int q = p; q >= 1; q >>= 1)
+#pragma unroll
+            for (int j = q % p; j + q < kK; j += 2 * q)
+#pragma unroll
+                for (int i = 0; i < q; ++i)
+                    if (i + j + q < kK && (i + j) / (2 * p) == (i + j + q) / (2 * p)) {
+                        const unsigned long long lo = key[i + j], hi = key[i + j + q];
+                        const bool swap = hi < lo;
+                        key[i + j] = swap ? hi : lo;
+                        key[i + j + q] = swap ? lo : hi;
+                    }
+#pragma unroll
+    for (int k = 0; k < kK; ++k) out[k] = (int32_t)(uint32_t)key[k];
+}
+
+// each(candidate) for the centres spos[rg.x, rg.y), loaded two at a time so that their latencies overlap.
+template <class Each>
+__device__ __forceinline__ void for_centres(uint2 rg, const float4 *spos, Each &&each) {
+    for (uint32_t q = rg.x; q < rg.y; q += 2) {
+        const float4 o0 = __ldg(spos + q), o1 = __ldg(spos + min(q + 1u, rg.y - 1u));
+        each(o0);
+        if (q + 1u < rg.y) each(o1);
+    }
+}
+
+// Lists of queries that would examine more than kQueryBudget centres: the best among the first
+// kQueryBudget in ring order (coincident or non-finite centres only; kept out of the kernels' registers).
+__device__ __noinline__ void ring_search_bounded(float4 p, const KnnGrid *gp, const uint32_t *starts, const float4 *spos,
+                                                 int32_t *out) {
+    float bd[kK];
+    uint32_t bi[kK];
+    ring_search(p, *gp, starts, spos, bd, bi);
+    for (int k = 0; k < kK; ++k) out[k] = (int32_t)bi[k];
+}
+
+// sqrt with a relative error below 2^-20 on the safe side, for windows of cells.
+__device__ __forceinline__ float sqrt_above(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y * (1.f + 1.f / 524288.f);
+}
+
+// The cells of a query point.
+struct CellPoint {
+    float4 p;
+    int cx, cy, cz;
+};
+
+// Squared distance from q.p to row (y, z) of cells across x; 0 across its own slabs, which may reach past
+// their box (an axis has at most 2,048 cells).
+__device__ __forceinline__ float row_gap(const CellPoint &q, const KnnGrid &G, int y, int z) {
+    const float gy = y == q.cy ? 0.f : slab_gap(G.lo[1], G.h, G.slack, q.p.y, y);
+    const float gz = z == q.cz ? 0.f : slab_gap(G.lo[2], G.h, G.slack, q.p.z, z);
+    return fmaf(gy, gy, gz * gz);
+}
+
+// The centres of the cells [x0, x1] of row (y, z) that lie within sqrt(left) of q.p along x.
+__device__ __forceinline__ uint2 row_within(const CellPoint &q, const KnnGrid &G, const uint32_t *starts, int y, int z,
+                                            int x0, int x1, float left) {
+    const float w = sqrt_above(left) + G.slack;
+    x0 = max(x0, min(cell_axis(q.p.x - w, G.lo[0], G.inv_h, G.dims[0]), q.cx));
+    x1 = min(x1, max(cell_axis(q.p.x + w, G.lo[0], G.inv_h, G.dims[0]), q.cx));
+    const int row = G.dims[0] * (y + G.dims[1] * z);
+    return row_range(starts, row + x0, row + x1);
+}
+
+// First pass: the 27 cells around q's, then further rings (at most `rings` in all) until bd holds 16
+// distances and the searched cells reach sqrt(reach) of the 16th in every open direction. The middle rows come
+// first, so that the bound soon leaves most of the others out. Returns whether bd holds 16 distances.
+__device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid &G, const uint32_t *starts,
+                                               const float4 *spos, int rings, float reach, uint32_t &examined,
+                                               float (&bd)[kK]) {
+    for (int R = 1; R <= rings && examined <= kQueryBudget; ++R) {
+        const int x0 = max(q.cx - R, 0), x1 = min(q.cx + R, G.dims[0] - 1);
+        for (int zi = 0; zi <= 2 * R; ++zi) {
+            const int z = q.cz + ((zi & 1) ? -((zi + 1) >> 1) : (zi >> 1));
+            if (z < 0 || z >= G.dims[2]) continue;
+            for (int yi = 0; yi <= 2 * R; ++yi) {
+                const int y = q.cy + ((yi & 1) ? -((yi + 1) >> 1) : (yi >> 1));
+                if (y < 0 || y >= G.dims[1]) continue;
+                const float left = bd[kK - 1] - row_gap(q, G, y, z);
+                if (left < 0.f) continue;
+                const bool inner = R > 1 && abs(z - q.cz) < R && abs(y - q.cy) < R;  // only the two x faces are new
+                for (int side = 0; side < (inner ? 2 : 1); ++side) {
+                    const int xa = !inner ? x0 : (side == 0 ? q.cx - R : q.cx + R), xb = !inner ? x1 : xa;
+                    if (xa < 0 || xb >= G.dims[0]) continue;
+                    const uint2 rg = row_within(q, G, starts, y, z, xa, xb, left);
+                    examined += rg.y - rg.x;
+                    if (examined > kQueryBudget) break;
+                    for_centres(rg, spos, [&](float4 o) { insert_dist(dist2(q.p, o), bd); });
+                }
+            }
+        }
+        const bool full = bd[kK - 1] < __int_as_float(0x7f800000);
+        float b = __int_as_float(0x7f800000);  // least distance to an open face of the searched cells
+        bool all = true;
+        auto face = [&](bool open, float g) {
+            if (open) { b = fminf(b, g); all = false; }
+        };
+        face(q.cx - R > 0, q.p.x - (G.lo[0] + (float)(q.cx - R) * G.h));
+        face(q.cx + R < G.dims[0] - 1, (G.lo[0] + (float)(q.cx + R + 1) * G.h) - q.p.x);
+        face(q.cy - R > 0, q.p.y - (G.lo[1] + (float)(q.cy - R) * G.h));
+        face(q.cy + R < G.dims[1] - 1, (G.lo[1] + (float)(q.cy + R + 1) * G.h) - q.p.y);
+        face(q.cz - R > 0, q.p.z - (G.lo[2] + (float)(q.cz - R) * G.h));
+        face(q.cz + R < G.dims[2] - 1, (G.lo[2] + (float)(q.cz + R + 1) * G.h) - q.p.z);
+        b = fmaxf(b, 0.f);
+        if (all || (full && reach * bd[kK - 1] <= b * b)) return full;
+    }
+    return bd[kK - 1] < __int_as_float(0x7f800000);
+}
+
+// Second pass: the centres within sqrt(bound) of q.p, from the rows of cells that the ball reaches.
+__device__ __forceinline__ void ball_centres(const CellPoint &q, const KnnGrid &G, const uint32_t *starts,
+                                             const float4 *spos, float bound, uint32_t &examined, Found &f) {
+    const float rad = sqrt_above(bound) + G.slack;
+    const int z0 = min(cell_axis(q.p.z - rad, G.lo[2], G.inv_h, G.dims[2]), q.cz),
+              z1 = max(cell_axis(q.p.z + rad, G.lo[2], G.inv_h, G.dims[2]), q.cz),
+              y0 = min(cell_axis(q.p.y - rad, G.lo[1], G.inv_h, G.dims[1]), q.cy),
+              y1 = max(cell_axis(q.p.y + rad, G.lo[1], G.inv_h, G.dims[1]), q.cy);
+    for (int z = z0; z <= z1; ++z)
+        for (int y = y0; y <= y1; ++y) {
+            const float left = bound - row_gap(q, G, y, z);
+            if (left < 0.f) continue;
+            const uint2 rg = row_within(q, G, starts, y, z, 0, G.dims[0] - 1, left);
+            examined += rg.y - rg.x;
+            if (examined > kQueryBudget) break;
+            for_centres(rg, spos, [&](float4 o) {
+                const float d = dist2(q.p, o);
+                if (d <= bound) add_found(f, d, __float_as_uint(o.w));
+            });
+        }
+}
+
+__device__ __forceinline__ CellPoint cell_point(float4 p, const KnnGrid &G) {
+    return CellPoint{p, cell_axis(p.x, G.lo[0], G.inv_h, G.dims[0]), cell_axis(p.y, G.lo[1], G.inv_h, G.dims[1]),
+                     cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2])};
+}
+
+__global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_query(const float4 *spos, const uint32_t *starts,
+                                                                         const KnnGrid *gp, int n, int32_t *knn) {
+    __shared__ uint2 s_found[kK][kQueryThreads];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const float4 p = spos[r];
-    float bd[kK];
-    uint32_t bi[kK];
-    ring_search(p, *gp, ranges, spos, bd, bi);
     int32_t *out = knn + (size_t)__float_as_uint(p.w) * kK;
+    const KnnGrid G = *gp;
+    const CellPoint q = cell_point(p, G);
+    float bd[kK];
 #pragma unroll
-    for (int k = 0; k < kK; ++k) out[k] = (int32_t)bi[k];
+    for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
+    uint32_t examined = 0;
+    near_distances(q, G, starts, spos, 1 << 20, kReach, examined, bd);
+    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
+    if (examined <= kQueryBudget) {
+        examined = 0;
+        ball_centres(q, G, starts, spos, bd[kK - 1], examined, f);
+    }
+    if (examined > kQueryBudget) {
+        ring_search_bounded(p, gp, starts, spos, out);
+        return;
+    }
+    int32_t idx[kK];
+    sorted_indices(f, idx);
+#pragma unroll
+    for (int k = 0; k < kK; ++k) out[k] = idx[k];
 }
 
 // Cell keys of query points (w = 0: no query, sorted after every cell).
@@ -381,28 +603,154 @@ __global__ void __launch_bounds__(256) k_knn_point_keys(const float4 *pts, int m
                                                    G.dims[1] * cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2])));
 }
 
+// Walks Chebyshev rings of 2 x 2 x 2-cell blocks around p's block as block_search does and calls
+// scan(range) for the centres of every row of a block's cells that lies within bound() of p. Stops after
+// the ring `rings`, or when the searched blocks enclose everything within bound(). Returns the last ring.
+template <class Bound, class Scan>
+__device__ __forceinline__ int block_walk(float4 p, const KnnGrid &G, const uint32_t *starts, const uint32_t *bcount,
+                                          int rings, Bound &&bound, Scan &&scan) {
+    const int dx = G.dims[0], dy = G.dims[1], dz = G.dims[2];
+    const int bx_n = block_dim(dx), by_n = block_dim(dy), bz_n = block_dim(dz);
+    const int cx = cell_axis(p.x, G.lo[0], G.inv_h, dx), cy = cell_axis(p.y, G.lo[1], G.inv_h, dy),
+              cz = cell_axis(p.z, G.lo[2], G.inv_h, dz);
+    const int cbx = cx >> 1, cby = cy >> 1, cbz = cz >> 1;
+    const float h = G.h, H = G.h + G.h, sl = G.slack;
+    const float lx = G.lo[0], ly = G.lo[1], lz = G.lo[2];
+    // no gap to p's own slab, which may reach past its box (an axis has at most 2,048 cells)
+    auto gap = [&](float lo, float w, float x, int i, int own) { return i == own ? 0.f : slab_gap(lo, w, sl, x, i); };
+    // distance from p to the grid's box along each axis
+    const float ox = fmaxf(fmaxf(lx - sl - p.x, p.x - (lx + (float)dx * h + sl)), 0.f);
+    const float oy = fmaxf(fmaxf(ly - sl - p.y, p.y - (ly + (float)dy * h + sl)), 0.f);
+    const float oz = fmaxf(fmaxf(lz - sl - p.z, p.z - (lz + (float)dz * h + sl)), 0.f);
+    int ring = 0;
+    for (;; ++ring) {
+        const int z0 = max(cbz - ring, 0), z1 = min(cbz + ring, bz_n - 1);
+        const int y0 = max(cby - ring, 0), y1 = min(cby + ring, by_n - 1);
+        const int x0 = max(cbx - ring, 0), x1 = min(cbx + ring, bx_n - 1);
+        auto visit = [&](int bx, int by, int bz, float gyz) {
+            const float gx = gap(lx, H, p.x, bx, cbx);
+            if (fmaf(gx, gx, gyz) > bound()) return;
+            if (__ldg(bcount + (bx + bx_n * (by + by_n * bz))) == 0u) return;
+            const int fz1 = min(2 * bz + 1, dz - 1), fy1 = min(2 * by + 1, dy - 1), fx1 = min(2 * bx + 1, dx - 1);
+            for (int fz = 2 * bz; fz <= fz1; ++fz) {
+                const float hz = gap(lz, h, p.z, fz, cz);
+                for (int fy = 2 * by; fy <= fy1; ++fy) {
+                    const float hy = gap(ly, h, p.y, fy, cy);
+                    const float hyz = fmaf(hy, hy, hz * hz);
+                    if (hyz > bound()) continue;
+                    int fa = 2 * bx, fb = fx1;
+                    const float ha = gap(lx, h, p.x, fa, cx), hb = gap(lx, h, p.x, fb, cx);
+                    if (fmaf(ha, ha, hyz) > bound()) ++fa;
+                    if (fmaf(hb, hb, hyz) > bound()) --fb;
+                    const int row = dx * (fy + dy * fz);
+                    scan(row_range(starts, row + fa, row + fb));
+                }
+            }
+        };
+        for (int bz = z0; bz <= z1; ++bz) {
+            const float gz = gap(lz, H, p.z, bz, cbz);
+            if (gz * gz > bound()) continue;
+            for (int by = y0; by <= y1; ++by) {
+                const float gy = gap(ly, H, p.y, by, cby);
+                const float gyz = fmaf(gy, gy, gz * gz);
+                if (gyz > bound()) continue;
+                if (abs(bz - cbz) < ring && abs(by - cby) < ring) {  // only the two x faces are new
+                    if (cbx - ring >= 0) visit(cbx - ring, by, bz, gyz);
+                    if (cbx + ring < bx_n) visit(cbx + ring, by, bz, gyz);
+                } else {
+                    for (int bx = x0; bx <= x1; ++bx) visit(bx, by, bz, gyz);
+                }
+            }
+        }
+        if (ring >= rings) break;
+        // least distance to the grid's box beyond the searched blocks' open faces
+        float b2 = __int_as_float(0x7f800000);
+        bool all = true;
+        auto face = [&](bool open, float g, float o1, float o2) {
+            if (!open) return;
+            g = fmaxf(g - sl, 0.f);
+            b2 = fminf(b2, fmaf(g, g, fmaf(o1, o1, o2 * o2)));
+            all = false;
+        };
+        face(cbx - ring > 0, p.x - (lx + (float)(cbx - ring) * H), oy, oz);
+        face(cbx + ring < bx_n - 1, (lx + (float)(cbx + ring + 1) * H) - p.x, oy, oz);
+        face(cby - ring > 0, p.y - (ly + (float)(cby - ring) * H), ox, oz);
+        face(cby + ring < by_n - 1, (ly + (float)(cby + ring + 1) * H) - p.y, ox, oz);
+        face(cbz - ring > 0, p.z - (lz + (float)(cbz - ring) * H), ox, oy);
+        face(cbz + ring < bz_n - 1, (lz + (float)(cbz + ring + 1) * H) - p.z, ox, oy);
+        if (all) break;
+        if (bound() < __int_as_float(0x7f800000) && bound() <= b2 * (1.f - 1.f / 1048576.f)) break;
+    }
+    return ring;
+}
+
+// As ring_search_bounded, for point queries.
+__device__ __noinline__ void block_search_bounded(float4 p, const KnnGrid *gp, const uint32_t *starts,
+                                                  const uint32_t *bcount, const float4 *spos, int32_t *out) {
+    float bd[kK];
+    uint32_t bi[kK];
+    block_search(p, *gp, starts, bcount, spos, bd, bi);
+    for (int k = 0; k < kK; ++k) out[k] = (int32_t)bi[k];
+}
+
 // Queries at arbitrary points, taken in cell order (order[r]: the r-th query by cell), so a
 // warp searches one neighbourhood; w = 0: no query, the list is all -1.
-__global__ void __launch_bounds__(32) k_knn_points(const float4 *spos, const uint2 *ranges, const uint32_t *bcount,
-                                                    const KnnGrid *gp, const float4 *pts, const uint32_t *order, int m,
-                                                    int32_t *knn) {
+__global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const float4 *spos, const uint32_t *starts,
+                                                                          const uint32_t *bcount, const KnnGrid *gp,
+                                                                          const float4 *pts, const uint32_t *order,
+                                                                          int m, int32_t *knn) {
+    __shared__ uint2 s_found[kK][kQueryThreads];
     const int r0 = blockIdx.x * blockDim.x + threadIdx.x;
     if (r0 >= m) return;
     const uint32_t r = __ldg(order + r0);
     const float4 p = pts[r];
-    float bd[kK];
-    uint32_t bi[kK];
+    int4 *out = reinterpret_cast<int4 *>(knn + (size_t)r * kK);
+    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
     if (p.w != 0.f) {
         const KnnGrid G = *gp;
-        block_search(p, G, ranges, bcount, spos, bd, bi);
-    } else {
+        float bd[kK];
 #pragma unroll
-        for (int k = 0; k < kK; ++k) bi[k] = 0xffffffffu;
+        for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
+        uint32_t examined = 0;
+        const CellPoint q = cell_point(p, G);
+        // most queries lie within a few cells of 16 centres; the others walk blocks, which skip empty space
+        const bool near = near_distances(q, G, starts, spos, kNearRings, kReach, examined, bd);
+        int rings = 0;
+        if (!near && examined <= kQueryBudget) {
+#pragma unroll
+            for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
+            examined = 0;
+            rings = block_walk(
+                p, G, starts, bcount, max(max(G.dims[0], G.dims[1]), G.dims[2]), [&]() { return bd[kK - 1]; },
+                [&](uint2 rg) {
+                    examined += rg.y - rg.x;
+                    if (examined > kQueryBudget) return;
+                    for_centres(rg, spos, [&](float4 o) { insert_dist(dist2(p, o), bd); });
+                });
+        }
+        const float bound = bd[kK - 1];
+        if (examined <= kQueryBudget) {
+            examined = 0;
+            if (near)
+                ball_centres(q, G, starts, spos, bound, examined, f);
+            else
+                block_walk(p, G, starts, bcount, rings, [&]() { return bound; },
+                           [&](uint2 rg) {
+                               for_centres(rg, spos, [&](float4 o) {
+                                   const float d = dist2(p, o);
+                                   if (d <= bound) add_found(f, d, __float_as_uint(o.w));
+                               });
+                           });
+        }
+        if (examined > kQueryBudget) {
+            block_search_bounded(p, gp, starts, bcount, spos, reinterpret_cast<int32_t *>(out));
+            return;
+        }
     }
-    int4 *out = reinterpret_cast<int4 *>(knn + (size_t)r * kK);
+    int32_t idx[kK];
+    sorted_indices(f, idx);
 #pragma unroll
-    for (int k = 0; k < kK; k += 4)
-        out[k / 4] = make_int4((int32_t)bi[k], (int32_t)bi[k + 1], (int32_t)bi[k + 2], (int32_t)bi[k + 3]);
+    for (int k = 0; k < kK; k += 4) out[k / 4] = make_int4(idx[k], idx[k + 1], idx[k + 2], idx[k + 3]);
 }
 
 // Cell sort of m query points, after the grid's own workspace.
@@ -451,20 +799,23 @@ static cudaError_t knn_build(int32_t n, const float4 *pos, void *workspace, cons
     KnnGrid *grid = at<KnnGrid>(workspace, L.grid);
     cudaError_t e = cudaMemsetAsync(bb, 0xff, 12, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 12, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(at<void>(workspace, L.ranges), 0, 8ull * L.cap_cells, s);
+    uint32_t *starts = at<uint32_t>(workspace, L.starts);
+    if (e == cudaSuccess) e = cudaMemsetAsync(starts, 0, 4ull * (L.cap_cells + 1ull), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(at<void>(workspace, L.bcount), 0, 4ull * L.cap_cells, s);
     if (e != cudaSuccess) return e;
     k_knn_bbox<<<min(ceil_div_u64(n, 256), 1024u), 256, 0, s>>>(pos, n, bb);
     k_knn_grid<<<1, 1, 0, s>>>(bb, L.cap_cells, grid);
     uint32_t *keys[2] = {at<uint32_t>(workspace, L.keys0), at<uint32_t>(workspace, L.keys1)};
     uint32_t *vals[2] = {at<uint32_t>(workspace, L.vals0), at<uint32_t>(workspace, L.vals1)};
-    k_knn_keys<<<ceil_div_u64(n, 256), 256, 0, s>>>(pos, n, grid, keys[0], at<uint32_t>(workspace, L.bcount));
+    k_knn_keys<<<ceil_div_u64(n, 256), 256, 0, s>>>(pos, n, grid, keys[0], starts, at<uint32_t>(workspace, L.bcount));
+    // cell counts -> first centre of each cell, and the end
+    e = exclusive_scan(starts, starts, L.cap_cells + 1u, at<uint32_t>(workspace, L.partials), nullptr, s);
+    if (e != cudaSuccess) return e;
     e = radix_sort(keys, vals, true, nullptr, (uint32_t)n, L.bits, at<uint32_t>(workspace, L.hist),
                    at<uint32_t>(workspace, L.partials), s);
     if (e != cudaSuccess) return e;
     const int res = ((L.bits + 7) / 8) & 1;
-    k_knn_ranges<<<ceil_div_u64(n, 256), 256, 0, s>>>(keys[res], vals[res], pos, n, at<uint2>(workspace, L.ranges),
-                                                     at<float4>(workspace, L.spos));
+    k_knn_gather<<<ceil_div_u64(n, 256), 256, 0, s>>>(vals[res], pos, n, at<float4>(workspace, L.spos));
     return cudaGetLastError();
 }
 
@@ -493,7 +844,7 @@ cudaError_t knn_points_run(int32_t n, const float4 *pos, int32_t m, const float4
     const int res = ((Q.bits + 7) / 8) & 1;
     // one warp per CTA: query walks differ widely in length, and a CTA of several warps would hold
     // its slot until its longest walk ended
-    k_knn_points<<<ceil_div_u64(m, 32), 32, 0, s>>>(at<float4>(workspace, L.spos), at<uint2>(workspace, L.ranges),
+    k_knn_points<<<ceil_div_u64(m, kQueryThreads), kQueryThreads, 0, s>>>(at<float4>(workspace, L.spos), at<uint32_t>(workspace, L.starts),
                                                      at<uint32_t>(workspace, L.bcount), at<KnnGrid>(workspace, L.grid),
                                                      pts, vals[res], m, knn);
     return cudaGetLastError();
@@ -512,7 +863,7 @@ extern "C" ges_status ges_knn(int32_t n, const float *pos_op, void *workspace, s
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float4 *pos = reinterpret_cast<const float4 *>(pos_op);
     if (knn_build(n, pos, workspace, L, s) != cudaSuccess) return GES_ERR_CUDA;
-    k_knn_query<<<ceil_div_u64(n, 128), 128, 0, s>>>(at<float4>(workspace, L.spos), at<uint2>(workspace, L.ranges),
+    k_knn_query<<<ceil_div_u64(n, kQueryThreads), kQueryThreads, 0, s>>>(at<float4>(workspace, L.spos), at<uint32_t>(workspace, L.starts),
                                                     at<KnnGrid>(workspace, L.grid), n, knn);
     return cudaGetLastError() == cudaSuccess ? GES_OK : GES_ERR_CUDA;
 }
