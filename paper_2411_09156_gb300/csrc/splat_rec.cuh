@@ -50,16 +50,22 @@ struct NbRec {
     int km;
 };
 
-__device__ __forceinline__ NbRec load_rec(const float4 *rec, int i) {
-    const float4 *r = rec + kRec * (size_t)i;
+__device__ __forceinline__ NbRec make_rec(float4 r0, float4 a, float4 b, float4 c, float4 d) {
     NbRec N;
-    N.r0 = __ldg(r);
-    const float4 a = __ldg(r + 1), b = __ldg(r + 2), c = __ldg(r + 3), d = __ldg(r + 4);
+    N.r0 = r0;
     N.R[0] = a.x; N.R[1] = a.y; N.R[2] = a.z; N.R[3] = a.w;
     N.R[4] = b.x; N.R[5] = b.y; N.R[6] = b.z; N.R[7] = b.w;
     N.R[8] = c.x; N.ia[0] = c.y; N.ia[1] = c.z; N.ia[2] = c.w;
     N.beta = d.x; N.smin = d.y; N.km = __float_as_int(d.z);
     return N;
 }
+
+__device__ __forceinline__ NbRec load_rec(const float4 *rec, int i) {
+    const float4 *r = rec + kRec * (size_t)i;
+    return make_rec(__ldg(r), __ldg(r + 1), __ldg(r + 2), __ldg(r + 3), __ldg(r + 4));
+}
+
+// A record staged in shared memory.
+__device__ __forceinline__ NbRec unpack_rec(const float4 (&r)[kRec]) { return make_rec(r[0], r[1], r[2], r[3], r[4]); }
 
 }  // namespace ges
