@@ -352,7 +352,7 @@ GES_API ges_status ges_knn(int32_t n, const float *pos_op, void *workspace, size
  *            query (its list is all -1)
  *   knn      [m, 16] int32 (written, 16-byte aligned): point j's neighbours by increasing
  *            distance, ties to the lower index
- * The points are searched in grid-cell order; cells are grouped in 2 x 2 x 2 blocks whose
+ * The points are searched in grid-cell order; cells are grouped in 4 x 4 x 4 blocks whose
  * counts let a query in empty space skip them. Exactness and the 65,536-candidate bound
  * are as for ges_knn. Workspace: ges_knn_points_workspace_bytes(n, m) bytes, 256-byte
  * aligned, no initialisation needed. n in [16, 2^26], m in [1, 2^28]. */

@@ -28,7 +28,11 @@ constexpr int kQueryThreads = 64, kQueryCtas = 16;
 // drops the few candidates too many, which costs less than another ring (reach 1: 1.61 ms against 1.42-1.45
 // at 0.25 and 0.5 for the centres; level-set queries 3.93 against 3.78 ms).
 constexpr float kReach = 0.25f;
-constexpr int kNearRings = 4;  // rings of cells that a point query tries before it walks blocks
+constexpr int kNearRings = 4;  // rings of cells that a point query tries before it walks blocks (2 and 3: within 5 %)
+// Blocks of 4 x 4 x 4 cells, with their point counts, let point queries skip empty space. Level-set queries of
+// five 1600x1040 views (whole call): 2.45-4.91 ms with 2 x 2 x 2 blocks, 2.53-3.28 with these, 2.63-3.69 with
+// 8 x 8 x 8.
+constexpr int kBlockShift = 2, kBlockSide = 1 << kBlockShift;
 
 struct KnnGrid {
     float lo[3];
@@ -150,8 +154,7 @@ __device__ __forceinline__ int cell_axis(float p, float lo, float inv_h, int dim
     return min(max(c, 0), dim - 1);
 }
 
-// Blocks of 2 x 2 x 2 cells, with their point counts, let point queries skip empty space.
-__device__ __forceinline__ int block_dim(int d) { return (d + 1) >> 1; }
+__device__ __forceinline__ int block_dim(int d) { return (d + kBlockSide - 1) >> kBlockShift; }
 
 __global__ void __launch_bounds__(256) k_knn_keys(const float4 *pos, int n, const KnnGrid *g, uint32_t *keys,
                                                   uint32_t *ccount, uint32_t *bcount) {
@@ -165,7 +168,8 @@ __global__ void __launch_bounds__(256) k_knn_keys(const float4 *pos, int n, cons
     const uint32_t cell = (uint32_t)(cx + G.dims[0] * (cy + G.dims[1] * cz));
     keys[i] = cell;
     atomicAdd(ccount + cell, 1u);
-    atomicAdd(bcount + ((cx >> 1) + block_dim(G.dims[0]) * ((cy >> 1) + block_dim(G.dims[1]) * (cz >> 1))), 1u);
+    atomicAdd(bcount + ((cx >> kBlockShift) + block_dim(G.dims[0]) * ((cy >> kBlockShift) +
+                        block_dim(G.dims[1]) * (cz >> kBlockShift))), 1u);
 }
 
 // The centres in cell order.
@@ -291,13 +295,11 @@ __device__ __forceinline__ float slab_gap(float lo, float w, float slack, float 
 }
 
 // The same search over Chebyshev rings of 2 x 2 x 2-cell blocks, for queries anywhere in
-// space (start points in front of a surface, rays past its edge): a block whose box lies
-// farther than the 16th candidate, or that holds no centre, costs one test and at most one
-// count read; the cells of the others are pruned and scanned as in ring_search.
-__device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const uint32_t *starts, const uint32_t *bcount,
-                                             const float4 *spos, float (&bd)[kK], uint32_t (&bi)[kK]) {
+// space: the order in which a query that exceeds the budget examines its centres.
+__device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const uint32_t *starts, const float4 *spos,
+                                             float (&bd)[kK], uint32_t (&bi)[kK]) {
     const int dx = G.dims[0], dy = G.dims[1], dz = G.dims[2];
-    const int bx_n = block_dim(dx), by_n = block_dim(dy), bz_n = block_dim(dz);
+    const int bx_n = (dx + 1) >> 1, by_n = (dy + 1) >> 1, bz_n = (dz + 1) >> 1;
     const int cbx = cell_axis(p.x, G.lo[0], G.inv_h, dx) >> 1, cby = cell_axis(p.y, G.lo[1], G.inv_h, dy) >> 1,
               cbz = cell_axis(p.z, G.lo[2], G.inv_h, dz) >> 1;
     const float h = G.h, H = G.h + G.h, sl = G.slack;
@@ -317,7 +319,6 @@ __device__ __forceinline__ void block_search(float4 p, const KnnGrid G, const ui
         auto visit = [&](int bx, int by, int bz, float gyz) {
             const float gx = slab_gap(lx, H, sl, p.x, bx);
             if (fmaf(gx, gx, gyz) > bd[kK - 1]) return;
-            if (__ldg(bcount + (bx + bx_n * (by + by_n * bz))) == 0u) return;
             const int fz1 = min(2 * bz + 1, dz - 1), fy1 = min(2 * by + 1, dy - 1), fx1 = min(2 * bx + 1, dx - 1);
             for (int fz = 2 * bz; fz <= fz1; ++fz) {
                 const float hz = slab_gap(lz, h, sl, p.z, fz);
@@ -530,6 +531,7 @@ __device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid
         face(q.cz + R < G.dims[2] - 1, (G.lo[2] + (float)(q.cz + R + 1) * G.h) - q.p.z);
         b = fmaxf(b, 0.f);
         if (all || (full && reach * bd[kK - 1] <= b * b)) return full;
+        if (R > 1 && R < rings && rings <= kNearRings && examined == 0u) return false;  // empty space: blocks skip it
     }
     return bd[kK - 1] < __int_as_float(0x7f800000);
 }
@@ -603,18 +605,18 @@ __global__ void __launch_bounds__(256) k_knn_point_keys(const float4 *pts, int m
                                                    G.dims[1] * cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2])));
 }
 
-// Walks Chebyshev rings of 2 x 2 x 2-cell blocks around p's block as block_search does and calls
-// scan(range) for the centres of every row of a block's cells that lies within bound() of p. Stops after
+// Walks Chebyshev rings of blocks around q's block and calls scan(range) for the centres of every row of
+// a block's cells that lies within bound() of q.p, cut to it along x: a block whose box lies farther, or
+// that holds no centre, costs one test and at most one count read. Stops after
 // the ring `rings`, or when the searched blocks enclose everything within bound(). Returns the last ring.
 template <class Bound, class Scan>
-__device__ __forceinline__ int block_walk(float4 p, const KnnGrid &G, const uint32_t *starts, const uint32_t *bcount,
+__device__ __forceinline__ int block_walk(const CellPoint &q, const KnnGrid &G, const uint32_t *starts, const uint32_t *bcount,
                                           int rings, Bound &&bound, Scan &&scan) {
     const int dx = G.dims[0], dy = G.dims[1], dz = G.dims[2];
     const int bx_n = block_dim(dx), by_n = block_dim(dy), bz_n = block_dim(dz);
-    const int cx = cell_axis(p.x, G.lo[0], G.inv_h, dx), cy = cell_axis(p.y, G.lo[1], G.inv_h, dy),
-              cz = cell_axis(p.z, G.lo[2], G.inv_h, dz);
-    const int cbx = cx >> 1, cby = cy >> 1, cbz = cz >> 1;
-    const float h = G.h, H = G.h + G.h, sl = G.slack;
+    const int cbx = q.cx >> kBlockShift, cby = q.cy >> kBlockShift, cbz = q.cz >> kBlockShift;
+    const float4 p = q.p;
+    const float h = G.h, H = (float)kBlockSide * G.h, sl = G.slack;
     const float lx = G.lo[0], ly = G.lo[1], lz = G.lo[2];
     // no gap to p's own slab, which may reach past its box (an axis has at most 2,048 cells)
     auto gap = [&](float lo, float w, float x, int i, int own) { return i == own ? 0.f : slab_gap(lo, w, sl, x, i); };
@@ -631,21 +633,14 @@ __device__ __forceinline__ int block_walk(float4 p, const KnnGrid &G, const uint
             const float gx = gap(lx, H, p.x, bx, cbx);
             if (fmaf(gx, gx, gyz) > bound()) return;
             if (__ldg(bcount + (bx + bx_n * (by + by_n * bz))) == 0u) return;
-            const int fz1 = min(2 * bz + 1, dz - 1), fy1 = min(2 * by + 1, dy - 1), fx1 = min(2 * bx + 1, dx - 1);
-            for (int fz = 2 * bz; fz <= fz1; ++fz) {
-                const float hz = gap(lz, h, p.z, fz, cz);
-                for (int fy = 2 * by; fy <= fy1; ++fy) {
-                    const float hy = gap(ly, h, p.y, fy, cy);
-                    const float hyz = fmaf(hy, hy, hz * hz);
-                    if (hyz > bound()) continue;
-                    int fa = 2 * bx, fb = fx1;
-                    const float ha = gap(lx, h, p.x, fa, cx), hb = gap(lx, h, p.x, fb, cx);
-                    if (fmaf(ha, ha, hyz) > bound()) ++fa;
-                    if (fmaf(hb, hb, hyz) > bound()) --fb;
-                    const int row = dx * (fy + dy * fz);
-                    scan(row_range(starts, row + fa, row + fb));
+            const int fz1 = min((bz + 1) << kBlockShift, dz), fy1 = min((by + 1) << kBlockShift, dy),
+                      fx1 = min((bx + 1) << kBlockShift, dx) - 1;
+            for (int fz = bz << kBlockShift; fz < fz1; ++fz)
+                for (int fy = by << kBlockShift; fy < fy1; ++fy) {
+                    const float left = bound() - row_gap(q, G, fy, fz);
+                    if (left < 0.f) continue;
+                    scan(row_within(q, G, starts, fy, fz, bx << kBlockShift, fx1, left));
                 }
-            }
         };
         for (int bz = z0; bz <= z1; ++bz) {
             const float gz = gap(lz, H, p.z, bz, cbz);
@@ -686,10 +681,10 @@ __device__ __forceinline__ int block_walk(float4 p, const KnnGrid &G, const uint
 
 // As ring_search_bounded, for point queries.
 __device__ __noinline__ void block_search_bounded(float4 p, const KnnGrid *gp, const uint32_t *starts,
-                                                  const uint32_t *bcount, const float4 *spos, int32_t *out) {
+                                                  const float4 *spos, int32_t *out) {
     float bd[kK];
     uint32_t bi[kK];
-    block_search(p, *gp, starts, bcount, spos, bd, bi);
+    block_search(p, *gp, starts, spos, bd, bi);
     for (int k = 0; k < kK; ++k) out[k] = (int32_t)bi[k];
 }
 
@@ -721,7 +716,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
             for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
             examined = 0;
             rings = block_walk(
-                p, G, starts, bcount, max(max(G.dims[0], G.dims[1]), G.dims[2]), [&]() { return bd[kK - 1]; },
+                q, G, starts, bcount, max(max(G.dims[0], G.dims[1]), G.dims[2]), [&]() { return bd[kK - 1]; },
                 [&](uint2 rg) {
                     examined += rg.y - rg.x;
                     if (examined > kQueryBudget) return;
@@ -734,7 +729,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
             if (near)
                 ball_centres(q, G, starts, spos, bound, examined, f);
             else
-                block_walk(p, G, starts, bcount, rings, [&]() { return bound; },
+                block_walk(q, G, starts, bcount, rings, [&]() { return bound; },
                            [&](uint2 rg) {
                                for_centres(rg, spos, [&](float4 o) {
                                    const float d = dist2(p, o);
@@ -743,7 +738,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
                            });
         }
         if (examined > kQueryBudget) {
-            block_search_bounded(p, gp, starts, bcount, spos, reinterpret_cast<int32_t *>(out));
+            block_search_bounded(p, gp, starts, spos, reinterpret_cast<int32_t *>(out));
             return;
         }
     }
