@@ -270,12 +270,13 @@ __device__ __forceinline__ float seg_sum(float x, int width) {
 // a lane keeps half of its values and adds its partner's copy of them, so 48 values cost
 // 24 + 12 + ... shuffles instead of 48 per level. 48 = 3 x 16 halves four times; with 32 lanes
 // the fifth level adds the 3 remaining values outright and the even lane of each pair writes.
-// Lane v writes the sums it holds, values [base, base + CNT), that exist (index < 3K). At the
+// Lane v writes the sums it holds, values [base, base + CNT), that exist (index < 3K), to `row`: its splat's
+// gradient, or (STAGED) its splat's row of the warp's staging table. At the
 // first level value 3k + c pairs with 3(k + 8) + c, both wc_c times a basis value, so the lane
 // takes Y_k and Y_k+8 in kept / sent order (16 selects) instead of swapping 24 product pairs.
-template <int SEG>
+template <int SEG, bool STAGED>
 __device__ __forceinline__ void write_sh_grad(const float (&wc)[3], const float (&Y)[16], int v, int K, bool ok,
-                                              float *gcol) {
+                                              float *row) {
     constexpr int HALVINGS = SEG >= 16 ? 4 : (SEG == 8 ? 3 : (SEG == 4 ? 2 : (SEG == 2 ? 1 : 0)));
     constexpr int CNT = 48 >> HALVINGS;
     float t[48];
@@ -310,10 +311,14 @@ __device__ __forceinline__ void write_sh_grad(const float (&wc)[3], const float 
 #pragma unroll
         for (int q = 0; q < CNT; ++q) t[q] += __shfl_xor_sync(0xffffffffu, t[q], 1);
     }
-    if (ok && (SEG < 32 || (v & 1) == 0)) {
+    if (STAGED && CNT % 4 == 0 && K == 16) {  // rows start at odd multiples of 16 bytes: no bank conflicts
+#pragma unroll
+        for (int q = 0; q + 3 < CNT; q += 4)
+            *reinterpret_cast<float4 *>(row + base + q) = make_float4(t[q], t[q + 1], t[q + 2], t[q + 3]);
+    } else if (ok && (SEG < 32 || (v & 1) == 0)) {
 #pragma unroll
         for (int q = 0; q < CNT; ++q)
-            if (base + q < K * 3) gcol[base + q] = t[q];
+            if (base + q < K * 3) row[base + q] = t[q];
     }
 }
 
@@ -560,7 +565,34 @@ __global__ void __launch_bounds__(32, 28) k_preprocess_bwd(PreBwdArgs a) {
     for (int k = 0; k < 16; ++k) Y[k] = 0.f;
     if (has) sh_eval(a.P.sh_degree, sdir[0], sdir[1], sdir[2], Y);
     // the 48 products wc_c Y_k summed over the segment's lanes
-    write_sh_grad<SEG>(wc, Y, v, K, splat_ok, a.g_color + (size_t)i * K * 3);
+    if (SEG > 1 || K <= 4) {
+        write_sh_grad<SEG, false>(wc, Y, v, K, splat_ok, a.g_color + (size_t)i * K3);
+        return;
+    }
+    // One view: a lane holds all of a splat's sums, and storing them itself wrote single floats 192 B apart. They
+    // are staged where the coefficients were (all lanes are past them) and stored by the warp in one run: 1.5M
+    // splats, SH3, 0.387 -> 0.160 ms; SH2, 0.254 -> 0.230. At SH1 (12 sums) and from 4 views on (12 sums or
+    // fewer a lane) the table costs as much as it saves; at 2 views it gains too (0.160 -> 0.111 ms at 800k),
+    // but the compiler then contracts the chain rule's products otherwise and moves its last bits.
+    __syncwarp();
+    write_sh_grad<SEG, true>(wc, Y, v, K, true, wsh + (lane / seg) * S);
+    __syncwarp();
+    {
+        const long long first = a.first + gw * spw;
+        const int nflt = (int)min((long long)spw, end - first) * K3;
+        float *dst = a.g_color + (size_t)first * K3;
+        if (K3 % 4 == 0 && ((uintptr_t)a.g_color & 15u) == 0) {
+            for (int q = lane; q < nflt / 4; q += 32) {
+                const int sp = 4 * q / K3;
+                reinterpret_cast<float4 *>(dst)[q] = *reinterpret_cast<const float4 *>(wsh + sp * S + (4 * q - sp * K3));
+            }
+        } else {
+            for (int q = lane; q < nflt; q += 32) {
+                const int sp = q / K3;
+                dst[q] = wsh[sp * S + (q - sp * K3)];
+            }
+        }
+    }
 }
 
 cudaError_t launch_preprocess(const PreArgs &a, cudaStream_t s) {
