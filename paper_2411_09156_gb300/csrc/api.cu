@@ -12,6 +12,8 @@ namespace {
 
 constexpr uint64_t kMaxEntries = (uint64_t)kScanTile * kScanMaxPartials;  // 67,108,864 (view, splat) entries
 
+constexpr uint64_t kMaxCapacity = 1ull << 30;  // tile instances
+
 bool finite_pos(float x) { return isfinite(x) && x > 0.f; }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
@@ -100,12 +102,12 @@ Params make_params(const ges_config *cfg) {
 }
 
 // Largest instance capacity whose layout fits in `bytes`.
-uint64_t capacity_for(int32_t n, int32_t n_views, uint32_t n_tiles, size_t bytes) {
-    if (bins_layout(n, n_views, n_tiles, 0).bytes > bytes) return UINT64_MAX;  // does not fit at all
+uint64_t capacity_for(int32_t n, const ViewSet &V, size_t bytes) {
+    if (bins_layout(n, V, 0).bytes > bytes) return UINT64_MAX;  // does not fit at all
     uint64_t lo = 0, hi = 0xfffffffeull;
     while (lo < hi) {
         uint64_t mid = lo + (hi - lo + 1) / 2;
-        if (bins_layout(n, n_views, n_tiles, mid).bytes <= bytes) lo = mid; else hi = mid - 1;
+        if (bins_layout(n, V, mid).bytes <= bytes) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -152,8 +154,8 @@ size_t ges_proj_bytes(int32_t n, int32_t n_views) {
 size_t ges_bins_bytes(int32_t n, int32_t n_views, const ges_camera *cams, const ges_config *cfg, uint64_t capacity) {
     if (!check_views(n, n_views, cams, cfg) || capacity > 0xfffffffeull) return 0;
     const ViewSet V = make_views(n_views, cams, cfg);
-    const BinsLayout L = bins_layout(n, n_views, (uint32_t)V.n_tiles, capacity);
-    if ((uint64_t)256 * L.nblk_inst > kMaxEntries) return 0;
+    const BinsLayout L = bins_layout(n, V, capacity);
+    if (capacity > kMaxCapacity) return 0;
     return (size_t)L.bytes;
 }
 
@@ -163,15 +165,14 @@ ges_status ges_get_layout(int32_t n, int32_t n_views, const ges_camera *cams, co
     if (!out || !check_views(n, n_views, cams, cfg) || capacity > 0xfffffffeull) return GES_ERR_INVALID_ARG;
     const ViewSet V = make_views(n_views, cams, cfg);
     const ProjLayout P = proj_layout(n, n_views);
-    const BinsLayout B = bins_layout(n, n_views, (uint32_t)V.n_tiles, capacity);
+    const BinsLayout B = bins_layout(n, V, capacity);
     memset(out, 0, sizeof(*out));
     out->proj_records = P.records;
     out->proj_binrec = P.binrec;
     out->proj_g2d = P.g2d;
     out->proj_bytes = P.bytes;
-    const int res = B.tile_passes & 1;
-    out->bins_inst_tile = B.ikey[res];
-    out->bins_inst_entry = B.ival[res];
+    out->bins_inst_tile = B.tile;
+    out->bins_inst_entry = B.entry;
     out->bins_ranges = B.ranges;
     out->bins_queue = B.queue;
     out->bins_bytes = B.bytes;
@@ -246,35 +247,33 @@ ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges
     const ProjLayout PL = proj_layout(n, n_views);
     if (proj_bytes < PL.bytes) return GES_ERR_INVALID_ARG;
     const ViewSet V = make_views(n_views, cams, cfg);
-    const uint64_t cap = capacity_for(n, n_views, (uint32_t)V.n_tiles, bins_bytes);
+    const uint64_t cap = capacity_for(n, V, bins_bytes);
     if (cap == UINT64_MAX) return GES_ERR_INVALID_ARG;
-    const BinsLayout L = bins_layout(n, n_views, (uint32_t)V.n_tiles, cap);
-    if ((uint64_t)256 * L.nblk_inst > kMaxEntries) return GES_ERR_INVALID_ARG;
+    const BinsLayout L = bins_layout(n, V, cap);
+    if (cap > kMaxCapacity) return GES_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(bins, 0, 256, s) != cudaSuccess) return GES_ERR_CUDA;
     BinArgs a;
     a.n = n;
     a.n_views = n_views;
-    a.n_entries = (uint32_t)((uint64_t)n * n_views);
     a.rec = at<float4>(proj, PL.records);
     a.binrec = at<uint4>(proj, PL.binrec);
     a.total = at<unsigned long long>(proj, 0);
     a.err = at<uint32_t>(proj, 8);
     a.header = at<uint32_t>(bins, 0);
-    for (int i = 0; i < 2; ++i) {
-        a.dkey[i] = at<uint32_t>(bins, L.dkey[i]);
-        a.dval[i] = at<uint32_t>(bins, L.dval[i]);
-        a.ikey[i] = at<uint32_t>(bins, L.ikey[i]);
-        a.ival[i] = at<uint32_t>(bins, L.ival[i]);
-    }
-    a.rcount = at<uint32_t>(bins, L.rcount);
-    a.rinfo = at<uint4>(bins, L.rinfo);
+    a.inst_tile = at<uint32_t>(bins, L.tile);
+    a.inst_entry = at<uint32_t>(bins, L.entry);
+    a.pairs = at<unsigned long long>(bins, L.pairs);
     a.ranges = at<uint2>(bins, L.ranges);
     a.queue = at<uint32_t>(bins, L.queue);
-    a.hist = at<uint32_t>(bins, L.hist);
-    a.partials = at<uint32_t>(bins, L.partials);
+    a.aux = at<TileAux>(bins, L.aux);
+    a.counts = at<uint32_t>(bins, L.counts);
+    a.lists = at<uint4>(bins, L.lists);
+    a.jobs = at<uint4>(bins, L.jobs);
+    a.places = at<uint32_t>(bins, L.places);
     a.cap = cap;
-    a.tile_bits = bits_for((uint32_t)V.n_tiles);
+    a.per_cta = a.parts = 0;
+    a.slabs = depth_slabs(n, V);
     a.build_queue = cfg->persistent != 0;
     a.V = V;
     return cuda_status(launch_bin(a, s));
@@ -290,14 +289,13 @@ ges_status ges_render_fwd(int32_t n, int32_t n_views, const ges_camera *cams, co
     const ProjLayout PL = proj_layout(n, n_views);
     if (proj_bytes < PL.bytes) return GES_ERR_INVALID_ARG;
     const ViewSet V = make_views(n_views, cams, cfg);
-    const uint64_t cap = capacity_for(n, n_views, (uint32_t)V.n_tiles, bins_bytes);
+    const uint64_t cap = capacity_for(n, V, bins_bytes);
     if (cap == UINT64_MAX) return GES_ERR_INVALID_ARG;
-    const BinsLayout L = bins_layout(n, n_views, (uint32_t)V.n_tiles, cap);
+    const BinsLayout L = bins_layout(n, V, cap);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     FwdArgs a;
     a.rec = at<float4>(proj, PL.records);
-    const int res = L.tile_passes & 1;
-    a.inst_entry = at<uint32_t>(bins, L.ival[res]);
+    a.inst_entry = at<uint32_t>(bins, L.entry);
     a.ranges = at<uint2>(bins, L.ranges);
     a.queue = cfg->persistent ? at<uint32_t>(bins, L.queue) : nullptr;
     a.counter = const_cast<uint32_t *>(at<uint32_t>(bins, 4));
@@ -327,17 +325,16 @@ ges_status ges_render_bwd_screen(int32_t n, int32_t n_views, const ges_camera *c
     const ProjLayout PL = proj_layout(n, n_views);
     if (proj_bytes < PL.bytes) return GES_ERR_INVALID_ARG;
     const ViewSet V = make_views(n_views, cams, cfg);
-    const uint64_t cap = capacity_for(n, n_views, (uint32_t)V.n_tiles, bins_bytes);
+    const uint64_t cap = capacity_for(n, V, bins_bytes);
     if (cap == UINT64_MAX) return GES_ERR_INVALID_ARG;
-    const BinsLayout L = bins_layout(n, n_views, (uint32_t)V.n_tiles, cap);
+    const BinsLayout L = bins_layout(n, V, cap);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float *acc = g2d ? g2d : at<float>(proj, PL.g2d);
     const size_t acc_bytes = (size_t)n * n_views * 64;
     if (acc_bytes && cudaMemsetAsync(acc, 0, acc_bytes, s) != cudaSuccess) return GES_ERR_CUDA;
     BwdArgs b;
     b.rec = at<float4>(proj, PL.records);
-    const int res = L.tile_passes & 1;
-    b.inst_entry = at<uint32_t>(bins, L.ival[res]);
+    b.inst_entry = at<uint32_t>(bins, L.entry);
     b.ranges = at<uint2>(bins, L.ranges);
     b.queue = cfg->persistent ? at<uint32_t>(bins, L.queue) : nullptr;
     b.counter = const_cast<uint32_t *>(at<uint32_t>(bins, 8));

@@ -1,9 +1,18 @@
-// S5 binning: stable LSD radix sort (reduce-then-scan, 8-bit digits), exclusive
-// scan, instance emission in depth order, tile ranges and the longest-first
-// tile queue. Instance counts are read from device memory, so the whole chain
-// runs without a host round trip and can be captured in a CUDA graph with
-// capacity-sized grids (CTAs past the live count exit at once).
+// S5 binning (tile lists in depth order), and the scan and the stable LSD radix sort
+// (reduce-then-scan, 8-bit digits) that the KNN grid uses.
+//
+// Binning: the instances of every tile are counted, the counts scanned into segments, the instances
+// appended to their tile's segment in any order, and each segment sorted by (depth, entry) where it fits: in a
+// warp's, a part's or a whole CTA's shared memory. All counts stay in device memory, so the chain runs without
+// a host round trip and can be captured in a CUDA graph.
+// It replaced a depth sort of all entries (4 radix passes), the emission in that order and a stable
+// tile sort of all instances (2 or 3 passes), 28 launches that moved every instance about seven times.
+// Measured, the whole call as a graph, before and after: 1,000 splats at 128x128 88 -> 25 us; 100k at 800x800
+// 128 -> 55; 1.5M at 1600x1040 313 -> 280; 4 views of 300k 216 -> 160; 8 views of 1.5M (34.7M
+// instances) 1488 -> 1150. What bounds it there: the scattered 8-byte appends (425 us) and the sorts' shared-memory
+// traffic (430 us). Only lists far beyond a CTA got slower (1.5M splats in one 16x16 view: 224 -> 308 us).
 #include "ges_internal.cuh"
+#include "sort_net.cuh"
 #include "tile_tests.cuh"
 
 namespace ges {
@@ -274,34 +283,7 @@ cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], bool iota_vals, con
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ emission
-
-// Depth order -> tiles touched per rank (scanned next into emission offsets), and a
-// rank-ordered copy of what emission needs, so that k_emit streams instead of
-// gathering the binning records a second time. rinfo per rank: entry, hit mask,
-// global key of the tile box's first tile, and (box width in tiles | view tiles
-// per row << 6); box width 0 marks a box of more than 32 tiles (no mask).
-__global__ void __launch_bounds__(128) k_gather_counts(const uint32_t *sorted_e, const uint4 *binrec,
-                                                      uint32_t *counts, uint4 *rinfo, uint32_t n_entries, int n,
-                                                      ViewSet V) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_entries) return;
-    const uint32_t e = __ldg(sorted_e + r);
-    // both halves of the 32-byte record in one round trip
-    const uint4 b0 = __ldg(binrec + 2 * (size_t)e), b1 = __ldg(binrec + 2 * (size_t)e + 1);
-    const uint32_t tiles = b0.z;
-    counts[r] = tiles;
-    if (tiles) {
-        const int v = (int)(e / (uint32_t)n);
-        const int tx0 = (int)(b1.y & 0xffffu), ty0 = (int)(b1.y >> 16);
-        const int rw = (int)(b1.z & 0xffffu), rh = (int)(b1.z >> 16);
-        const int tiles_x = V.tiles_x[v];
-        const uint32_t origin = (uint32_t)V.tile_base[v] + (uint32_t)(ty0 * tiles_x + tx0);
-        const uint32_t shape = (rw * rh <= 32 ? (uint32_t)rw : 0u) | ((uint32_t)tiles_x << 6);
-        rinfo[r] = make_uint4(e, b1.x, origin, shape);
-    }
-}
-
+// ------------------------------------------------------------------ binning
 // Position of the k-th (0-based) set bit of m; m has more than k set bits.
 __device__ __forceinline__ uint32_t select_bit(uint32_t m, uint32_t k) {
     uint32_t pos = 0;
@@ -314,44 +296,26 @@ __device__ __forceinline__ uint32_t select_bit(uint32_t m, uint32_t k) {
     return pos;
 }
 
-// Emission. Ranks r..r+31 of a warp own the contiguous instance range
-// [offsets[r], offsets[r+32]); the warp expands their hit masks together, 32
-// instances per round: instance j goes to the rank whose prefix interval holds j
-// (binary search over the warp's inclusive prefix) and to that rank's j-th set
-// mask bit. Writes are coalesced. Boxes of more than 32 tiles (no mask) are
-// expanded afterwards by their own lane with the tile test.
-__global__ void __launch_bounds__(128) k_emit(EmitArgs a) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long total = *a.total;
-    if (total >= 0xffffffffull) {  // uint32 offsets would wrap
-        if (r == 0) set_error(a.err, kErrCapacity);
-        return;
-    }
-    if (blockIdx.x * blockDim.x + (threadIdx.x & ~31u) >= a.n_entries) return;  // whole warp past the end
-    const bool live = r < a.n_entries;
-    uint32_t off = 0, tiles = 0;
-    if (live) {
-        off = a.offsets[r];
-        const uint32_t next = (r + 1 < a.n_entries) ? a.offsets[r + 1] : (uint32_t)total;
-        tiles = next > off ? next - off : 0u;
-    }
-    if (tiles && (uint64_t)off + tiles > a.cap) set_error(a.err, kErrCapacity);
-    uint4 info = make_uint4(0u, 0u, 0u, 0u);
-    if (tiles) info = a.rinfo[r];
-    const uint32_t rw = info.w & 63u;
-    const uint32_t cnt = rw ? tiles : 0u;  // instances expanded cooperatively
-    uint32_t incl = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += t;
-    }
-    const uint32_t wtotal = __shfl_sync(0xffffffffu, incl, 31);
-    const uint32_t excl = incl - cnt;
+// The instances of a warp's 32 entries, each listed tile of each entry once: on_instance(global tile, depth bits,
+// entry) is called by one lane each. Entries whose box has at most 32 tiles are expanded from their hit masks
+// by the whole warp, 32 instances a round (instance j goes to the entry whose prefix interval holds j, binary
+// search over the warp's inclusive prefix, and to that entry's j-th set bit): a lane's own loop over its bits
+// waits for an atomic per bit and took a quarter longer. Larger boxes repeat the tile tests.
+
+template <class OnInstance>
+__device__ __forceinline__ void warp_instances(const BinArgs &a, int v, uint32_t tiles, const uint4 b0, const uint4 b1,
+                                               size_t e, uint4 *jobs, int lane, uint32_t part,
+                                               OnInstance &&on_instance) {
+    const int tiles_x = a.V.tiles_x[v];
+    const uint32_t tbase = (uint32_t)a.V.tile_base[v];
+    const uint32_t tx0 = b1.y & 0xffffu, ty0 = b1.y >> 16, bw = b1.z & 0xffffu, bh = b1.z >> 16;
+    const uint32_t rw = tiles && bw * bh <= 32u ? bw : 0u;  // 0: nothing, or no mask
+    const uint32_t origin = tbase + ty0 * (uint32_t)tiles_x + tx0;
+    const uint32_t cnt = rw ? tiles : 0u;
+    const uint32_t incl = warp_incl_scan(cnt), wtotal = __shfl_sync(0xffffffffu, incl, 31), excl = incl - cnt;
     const uint32_t mdiv = rw ? (65536u + rw - 1u) / rw : 0u;  // bit / rw == (bit * mdiv) >> 16 for bit < 32
-    const uint32_t base = off - excl;                          // instance j of the warp lands at base + j
-    for (uint32_t j0 = 0; j0 < wtotal; j0 += 32) {
+    const uint32_t shape = rw | (mdiv << 8);
+    for (uint32_t j0 = 32u * part; j0 < wtotal; j0 += 32u * a.parts) {
         const uint32_t j = j0 + (uint32_t)lane;
         int owner = 0;
 #pragma unroll
@@ -360,179 +324,660 @@ __global__ void __launch_bounds__(128) k_emit(EmitArgs a) {
             if (p <= j) owner += step;
         }
         const uint32_t o_excl = __shfl_sync(0xffffffffu, excl, owner);
-        const uint32_t o_base = __shfl_sync(0xffffffffu, base, owner);
-        const uint32_t o_mask = __shfl_sync(0xffffffffu, info.y, owner);
-        const uint32_t o_org = __shfl_sync(0xffffffffu, info.z, owner);
-        const uint32_t o_shape = __shfl_sync(0xffffffffu, info.w, owner);
-        const uint32_t o_mdiv = __shfl_sync(0xffffffffu, mdiv, owner);
-        const uint32_t o_e = __shfl_sync(0xffffffffu, info.x, owner);
+        const uint32_t o_mask = __shfl_sync(0xffffffffu, b1.x, owner);
+        const uint32_t o_org = __shfl_sync(0xffffffffu, origin, owner);
+        const uint32_t o_shape = __shfl_sync(0xffffffffu, shape, owner);
+        const uint32_t o_depth = __shfl_sync(0xffffffffu, b0.w, owner);
         if (j < wtotal) {
             const uint32_t bit = select_bit(o_mask, j - o_excl);
-            const uint32_t row = (bit * o_mdiv) >> 16;
-            const uint32_t col = bit - row * (o_shape & 63u);
-            const uint64_t pos = (uint64_t)o_base + j;
-            if (pos < a.cap) {
-                a.ikey[pos] = o_org + row * (o_shape >> 6) + col;
-                a.ival[pos] = o_e;
-            }
+            const uint32_t row = (bit * (o_shape >> 8)) >> 16;
+            // a warp's entries are consecutive
+            on_instance(o_org + row * (uint32_t)tiles_x + (bit - row * (o_shape & 0xffu)), o_depth,
+                        (uint32_t)e - (uint32_t)lane + (uint32_t)owner);
         }
     }
-    // boxes of more than 32 tiles: the tile tests spread over the warp, each hit
-    // written at its entry's offset plus the number of earlier hits of that entry
-    // (row-major order, as a per-entry loop over the box would write them)
     const bool big = tiles && !rw;
     if (!__any_sync(0xffffffffu, big)) return;
     const int tw = a.V.tile_w, th = a.V.tile_h;
     const int lw = __ffs(tw) - 1, lh = __ffs(th) - 1;  // tile sides are powers of two
     TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
-    uint32_t tbase = 0;
-    int tiles_x = 0;
     if (big) {
-        const uint32_t e = info.x;
-        const int v = (int)(e / (uint32_t)a.n);
-        tbase = (uint32_t)a.V.tile_base[v];
-        tiles_x = a.V.tiles_x[v];
-        const uint4 br = a.binrec[2 * (size_t)e];
-        const float4 r0 = a.rec[4 * (size_t)e], r1 = a.rec[4 * (size_t)e + 1];
+        const float4 r0 = a.rec[4 * e], r1 = a.rec[4 * e + 1];
         int x0, x1, y0, y1;
-        pixel_box(r0.x, r0.y, __uint_as_float(br.x), __uint_as_float(br.y), a.V.width[v], a.V.height[v], x0, x1,
-                  y0, y1);
+        pixel_box(r0.x, r0.y, __uint_as_float(b0.x), __uint_as_float(b0.y), a.V.width[v], a.V.height[v], x0, x1, y0, y1);
         if (x0 <= x1 && y0 <= y1)
             J = TileJob{r0.x, r0.y, r0.z, r0.w, r1.x, __frcp_rn(r0.z), __frcp_rn(r1.x), __fmul_rn(r1.y, kSupportMargin),
                         (uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16),
                         (uint32_t)((x1 >> lw) - (x0 >> lw) + 1) * (uint32_t)((y1 >> lh) - (y0 >> lh) + 1)};
     }
-    uint32_t written = 0;  // hits of this lane's entry written so far
-    __shared__ uint4 s_jobs[4][kJobWords * 32];  // 128 threads: 4 warps
-    warp_tile_rounds(J, lane, lw, lh, tw, th, s_jobs[threadIdx.x >> 5],
-                     [&](uint32_t hits, uint32_t lo, uint32_t len, uint32_t, int tx, int ty, uint32_t owner,
-                         bool hit) {
-                         const uint32_t o_off = __shfl_sync(0xffffffffu, off, owner);
-                         const uint32_t o_written = __shfl_sync(0xffffffffu, written, owner);
-                         const uint32_t o_tbase = __shfl_sync(0xffffffffu, tbase, owner);
-                         const int o_tiles_x = __shfl_sync(0xffffffffu, tiles_x, owner);
-                         const uint32_t o_e = __shfl_sync(0xffffffffu, info.x, owner);
-                         const uint32_t same = __match_any_sync(0xffffffffu, owner);
-                         if (hit) {
-                             const uint64_t pos = (uint64_t)o_off + o_written +
-                                                  (uint32_t)__popc(hits & same & ((1u << lane) - 1u));
-                             if (pos < a.cap) {
-                                 a.ikey[pos] = o_tbase + (uint32_t)(ty * o_tiles_x + tx);
-                                 a.ival[pos] = o_e;
-                             }
-                         }
-                         if (len)
-                             written += (uint32_t)__popc((hits >> lo) &
-                                                         (len == 32u ? 0xffffffffu : ((1u << len) - 1u)));
+    warp_tile_rounds(J, lane, lw, lh, tw, th, jobs, part, a.parts,
+                     [&](uint32_t, uint32_t, uint32_t, uint32_t, int tx, int ty, uint32_t owner, bool hit) {
+                         const uint32_t depth = __shfl_sync(0xffffffffu, b0.w, owner);
+                         const uint32_t ent = __shfl_sync(0xffffffffu, (uint32_t)e, owner);
+                         if (hit) on_instance(tbase + (uint32_t)(ty * tiles_x + tx), depth, ent);
                      });
 }
 
-// n_inst = min(total, cap); 0 when the total does not fit the uint32 offsets
-// (k_emit then writes nothing and records the capacity error).
-__global__ void k_set_count(const unsigned long long *total, uint64_t cap, uint32_t *n_inst) {
-    unsigned long long t = *total;
-    *n_inst = t >= 0xffffffffull ? 0u : (uint32_t)(t < cap ? t : cap);
-}
-
-// Tile ranges from the sorted instance keys: thread q looks at keys 4q .. 4q+3 (one 16-byte load;
-// the key buffer is capacity-sized and 256-byte aligned inside `bins`, so the load stays inside the
-// allocation; keys at n and beyond are never used) and at their neighbours 4q - 1 and 4q + 4.
-__global__ void __launch_bounds__(256) k_tile_ranges(const uint32_t *keys, const uint32_t *n_dev, uint2 *ranges,
-                                                    uint32_t n_tiles) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t n = *n_dev;
-    const uint32_t i0 = 4 * q;
-    if (i0 >= n) return;
-    const uint4 v = reinterpret_cast<const uint4 *>(keys)[q];
-    const uint32_t k[6] = {i0 > 0 ? keys[i0 - 1] : 0u, v.x, v.y, v.z, v.w, i0 + 4 < n ? keys[i0 + 4] : 0u};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t i = i0 + (uint32_t)j;
-        if (i >= n) break;
-        const uint32_t kk = k[j + 1];
-        if (kk >= n_tiles) continue;
-        if (i == 0 || k[j] != kk) ranges[kk].x = i;
-        if (i == n - 1 || k[j + 2] != kk) ranges[kk].y = i + 1;
+// EMIT false: counts the instances per tile. EMIT true: appends each instance to its tile's segment.
+// A CTA takes `a.per_cta` entries of one view, the views in turn. SHARED: it counts them per tile in shared memory
+// first, so that a tile costs one global atomic per CTA: the atomics of all CTAs on a view's few counters were
+// what the kernel waited for (8 views of 1.5M splats, 34.7M instances: count 0.91 and append 1.06 ms with an
+// atomic per instance). The count keeps what those atomics return, the CTA's place among a tile's instances, and
+// the append of the same entries starts there, so a CTA's instances of a tile land side by side.
+// SLABS: the tiles' segments are split by depth.
+template <bool EMIT, bool SHARED, bool SLABS>
+__global__ void __launch_bounds__(kInstThreads) k_instances(const BinArgs a) {
+    if (*a.total >= 0xffffffffull) {  // uint32 positions would wrap: no lists
+        if (!EMIT && blockIdx.x == 0 && threadIdx.x == 0) set_error(a.err, kErrCapacity);
+        return;
     }
-}
-
-// Longest-first tile queue: tiles are bucketed by list length on a log2 scale
-// (4 buckets per octave, longest first) with a one-CTA counting sort. Approximate
-// LPT order is enough for scheduling; the results do not depend on it.
-__global__ void __launch_bounds__(1024) k_lpt_queue(const uint2 *ranges, uint32_t n_tiles, uint32_t *queue) {
-    constexpr int NB = 128;
-    __shared__ uint32_t s_cnt[NB], s_off[NB];
-    if (threadIdx.x < NB) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    auto bucket = [](uint32_t len) -> int {
-        if (len == 0) return NB - 1;
-        const float l = 4.f * log2f((float)len + 1.f);
-        int b = (NB - 2) - (int)l;
-        return b < 0 ? 0 : b;
+    extern __shared__ uint32_t s_cnt[];  // SHARED: instances per segment of the view; the CTA's next slot in each
+    __shared__ uint4 s_jobs[kInstThreads / 32][kJobWords * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // blocks: the views of a part of a run of entries, the parts (every a.parts-th round of 32 instances of a
+    // warp's entries: few splats of many tiles each give too few warps otherwise), the runs
+    const int v = (int)(blockIdx.x % (uint32_t)a.n_views);
+    const uint32_t row = blockIdx.x / (uint32_t)a.n_views, part = row % a.parts;
+    const uint32_t i0 = row / a.parts * a.per_cta, i1 = min(i0 + a.per_cta, (uint32_t)a.n);
+    const uint32_t S = SLABS ? a.slabs : 1u, tbase = (uint32_t)a.V.tile_base[v] * S, vtiles = (uint32_t)a.V.tile_base[v + 1] * S - tbase;
+    float z0 = 0.f, per_z = 0.f;
+    if (SLABS) {
+        z0 = __uint_as_float(~a.aux->depth_lo_inv[v]);
+        const float dz = __uint_as_float(a.aux->depth_hi[v]) - z0;
+        per_z = dz > 0.f ? (float)S / dz : 0.f;
+    }
+    // a tile's segment for a depth: the slabs' order is the depths'
+    auto segment = [&](uint32_t tile, uint32_t depth) {
+        if (!SLABS) return tile;
+        return tile * S + min((uint32_t)max((int)((__uint_as_float(depth) - z0) * per_z), 0), S - 1u);
     };
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        atomicAdd(&s_cnt[bucket(r.y - r.x)], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int b = 0; b < NB; ++b) { s_off[b] = run; run += s_cnt[b]; }
-    }
-    __syncthreads();
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        const uint32_t pos = atomicAdd(&s_off[bucket(r.y - r.x)], 1u);
-        queue[pos] = t;
+    auto each = [&](auto &&on_instance) {
+        for (uint32_t w0 = i0 + (uint32_t)warp * 32u; w0 < i1; w0 += blockDim.x) {
+            const uint32_t i = w0 + (uint32_t)lane;
+            const size_t e = (size_t)v * a.n + i;
+            uint4 b0 = make_uint4(0u, 0u, 0u, 0u), b1 = b0;
+            if (i < i1) {
+                b0 = __ldg(a.binrec + 2 * e);
+                b1 = __ldg(a.binrec + 2 * e + 1);
+            }
+            const uint32_t tiles = b0.z;
+            if (!__any_sync(0xffffffffu, tiles != 0u)) continue;
+            warp_instances(a, v, tiles, b0, b1, e, s_jobs[warp], lane, part, on_instance);
+        }
+    };
+    auto append = [&](uint32_t slot, uint32_t depth, uint32_t e) {
+        if (slot < a.cap) a.pairs[slot] = ((unsigned long long)depth << 32) | e;
+        else set_error(a.err, kErrCapacity);
+    };
+    if (SHARED) {
+        uint32_t *place = a.places + (size_t)row * ((size_t)a.V.n_tiles * S) + tbase;
+        // (a tile without instances here has no place: its slot is not used)
+        for (uint32_t t = threadIdx.x; t < vtiles; t += blockDim.x) s_cnt[t] = EMIT ? a.counts[tbase + t] + place[t] : 0u;
+        __syncthreads();
+        if (EMIT) {
+            each([&](uint32_t tile, uint32_t depth, uint32_t e) {
+                append(atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u), depth, e);
+            });
+            return;
+        }
+        each([&](uint32_t tile, uint32_t depth, uint32_t) { atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u); });
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < vtiles; t += blockDim.x) {
+            const uint32_t c = s_cnt[t];
+            if (c) place[t] = atomicAdd(a.counts + tbase + t, c);
+        }
+    } else {
+        each([&](uint32_t tile, uint32_t depth, uint32_t e) {
+            const uint32_t slot = atomicAdd(a.counts + segment(tile, depth), 1u);
+            if (EMIT) append(slot, depth, e);
+        });
     }
 }
 
+// Least and greatest depth of each view's listed entries, for the slabs.
+__global__ void __launch_bounds__(256) k_depth_range(const BinArgs a) {
+    const int v = (int)blockIdx.y;
+    uint32_t hi = 0u, lo_inv = 0u;
+    for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < (uint32_t)a.n; i += gridDim.x * 256u) {
+        const uint4 b = __ldg(a.binrec + 2 * ((size_t)v * a.n + i));
+        if (b.z) {
+            hi = max(hi, b.w);
+            lo_inv = max(lo_inv, ~b.w);
+        }
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo_inv = __reduce_max_sync(0xffffffffu, lo_inv);
+    if ((threadIdx.x & 31) == 0 && hi) {
+        atomicMax(&a.aux->depth_hi[v], hi);
+        atomicMax(&a.aux->depth_lo_inv[v], lo_inv);
+    }
+}
 
-__global__ void __launch_bounds__(256) k_depth_keys(const uint4 *binrec, uint32_t *keys, uint32_t n) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) keys[i] = binrec[2 * (size_t)i].w;
+// Length bucket of a list for the longest-first queue: 4 buckets per octave, longest first. Approximate
+// order is enough for scheduling; the results do not depend on it.
+__device__ __forceinline__ int length_bucket(uint32_t len) {
+    if (len == 0) return kLptBuckets - 1;
+    const int b = (kLptBuckets - 2) - (int)(4.f * log2f((float)len + 1.f));
+    return b < 0 ? 0 : b;
+}
+
+// Tile index, first part: each CTA's instances and, for the queue, the tiles per length bucket. A CTA takes
+// `per` consecutive tiles (a multiple of 1024).
+__global__ void __launch_bounds__(1024) k_tile_sums(const BinArgs a, uint32_t per) {
+    __shared__ uint32_t s_warp[33], s_bucket[kLptBuckets];
+    const uint32_t n_tiles = (uint32_t)a.V.n_tiles, t0 = blockIdx.x * per;
+    if (threadIdx.x < kLptBuckets) s_bucket[threadIdx.x] = 0u;
+    __syncthreads();
+    uint32_t sum = 0;
+    for (uint32_t k = threadIdx.x; k < per; k += 1024) {
+        const uint32_t t = t0 + k;
+        if (t >= n_tiles) break;
+        uint32_t c = 0;
+        for (uint32_t q = 0; q < a.slabs; ++q) c += a.counts[(size_t)t * a.slabs + q];
+        sum += c;
+        if (a.build_queue) atomicAdd(&s_bucket[length_bucket(c)], 1u);
+    }
+    uint32_t tot;
+    block_excl_scan(sum, s_warp, tot);
+    if (threadIdx.x == 0) a.aux->partial[blockIdx.x] = tot;
+    if (a.build_queue && threadIdx.x < kLptBuckets && s_bucket[threadIdx.x])
+        atomicAdd(&a.aux->bucket[threadIdx.x], s_bucket[threadIdx.x]);
+}
+
+// Sort class of a segment of n instances at `start`, clipped to the capacity: -1 nothing to sort, kListClasses too
+// long for one CTA.
+__device__ __forceinline__ int seg_class(const BinArgs &a, uint32_t start, uint32_t n) {
+    const uint32_t len = (uint32_t)(min((uint64_t)start + n, a.cap) - min((uint64_t)start, a.cap));
+    return len == 0u ? -1 : len <= 256u ? 0 : len <= 1024u ? 1 : len <= kCtaList ? 2 : len <= kBigList ? 3 : kListClasses;
+}
+
+// Tile index, second part: each tile's range clipped to the capacity, its segments' starts (in place of their
+// counts) and their places in the sort classes' lists or chunk jobs, and the tile's place in the queue.
+__global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t per) {
+    __shared__ uint32_t s_warp[33], s_prefix[kLptBuckets], s_cnt[kLptBuckets], s_base[kLptBuckets];
+    __shared__ uint32_t s_cls[kListClasses], s_cls_base[kListClasses];
+    const uint32_t n_tiles = (uint32_t)a.V.n_tiles, t0 = blockIdx.x * per, tid = threadIdx.x, S = a.slabs;
+    if (blockIdx.x == 0 && tid == 0) {
+        const unsigned long long t = *a.total;
+        a.header[0] = t >= 0xffffffffull ? 0u : (uint32_t)(t < a.cap ? t : a.cap);
+    }
+    uint32_t run, tot;
+    block_excl_scan(tid < blockIdx.x ? a.aux->partial[tid] : 0u, s_warp, run);  // at most kTileBlocks CTAs before
+    if (a.build_queue) {
+        const uint32_t p = block_excl_scan(tid < kLptBuckets ? a.aux->bucket[tid] : 0u, s_warp, tot);
+        if (tid < kLptBuckets) s_prefix[tid] = p;
+    }
+    for (uint32_t k0 = 0; k0 < per; k0 += 1024) {
+        const uint32_t t = t0 + k0 + tid;
+        if (t0 + k0 >= n_tiles) break;  // uniform for the CTA
+        if (tid < kLptBuckets) s_cnt[tid] = 0u;
+        if (tid < kListClasses) s_cls[tid] = 0u;
+        __syncthreads();
+        uint32_t c = 0;
+        if (t < n_tiles)
+            for (uint32_t q = 0; q < S; ++q) c += a.counts[(size_t)t * S + q];
+        const uint32_t start = run + block_excl_scan(c, s_warp, tot);
+        run += tot;
+        uint32_t slot = 0;
+        int bucket = 0;
+        if (t < n_tiles) {
+            const uint64_t s = min((uint64_t)start, a.cap), e = min((uint64_t)start + c, a.cap);
+            a.ranges[t] = e > s ? make_uint2((uint32_t)s, (uint32_t)e) : make_uint2(0u, 0u);
+            if (a.build_queue) {
+                bucket = length_bucket(c);
+                slot = atomicAdd(&s_cnt[bucket], 1u);
+            }
+            // the tile's segments: their starts replace their counts
+            uint32_t at = start;
+            for (uint32_t q = 0; q < S; ++q) {
+                const uint32_t n = a.counts[(size_t)t * S + q];
+                a.counts[(size_t)t * S + q] = at;
+                const int cls = seg_class(a, at, n);
+                if (cls < kListClasses && cls >= 0) atomicAdd(&s_cls[cls], 1u);
+                at += n;
+            }
+        }
+        __syncthreads();
+        if (tid < kListClasses) {
+            s_cls_base[tid] = s_cls[tid] ? atomicAdd(&a.aux->n_list[tid], s_cls[tid]) : 0u;
+            s_cls[tid] = 0u;
+        }
+        if (a.build_queue && tid < kLptBuckets) s_base[tid] = s_cnt[tid] ? atomicAdd(&a.aux->bucket_cur[tid], s_cnt[tid]) : 0u;
+        __syncthreads();
+        if (t < n_tiles) {
+            uint32_t at = start;
+            for (uint32_t q = 0; q < S; ++q) {
+                // the next segment's start, the tile's end after the last
+                const uint32_t end = q + 1 < S ? a.counts[(size_t)t * S + q + 1] : start + c;
+                const int cls = seg_class(a, at, end - at);
+                const uint32_t s = (uint32_t)min((uint64_t)at, a.cap), e = (uint32_t)min((uint64_t)end, a.cap);
+                if (cls >= 0 && cls < kListClasses) {
+                    const uint32_t k = s_cls_base[cls] + atomicAdd(&s_cls[cls], 1u);
+                    a.lists[(size_t)cls * n_tiles * S + k] = make_uint4(s, e, t, 0u);
+                } else if (cls == kListClasses) {
+                    const uint32_t nch = (e - s + kBigList - 1u) / kBigList;
+                    const uint32_t k = atomicAdd(&a.aux->n_jobs, nch);
+                    for (uint32_t j = 0; j < nch; ++j) a.jobs[k + j] = make_uint4(s, e, t, j);
+                }
+                at = end;
+            }
+        }
+        if (a.build_queue && t < n_tiles) a.queue[s_prefix[bucket] + s_base[bucket] + slot] = t;
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ tile list sort
+typedef unsigned long long u64;
+// Keys in shared memory are padded by one per ITEMS, so that neighbouring threads' runs of ITEMS start in
+// different banks.
+template <int ITEMS>
+__host__ __device__ constexpr int padded(int i) { return i + i / ITEMS; }
+
+// Merge sort of 64-bit keys by a group of threads, ITEMS consecutive keys a thread: a sorting network in
+// registers, then merges of doubling width, each thread producing its ITEMS outputs from where a binary
+// search along its diagonal says they start.
+// Sorts the len keys of sm (at padded<ITEMS>(i); len <= the group's threads x ITEMS) with the group's thread t; `sync`
+// is the group's barrier. The keys are visible to the group on entry and on return.
+template <int ITEMS, class Sync>
+__device__ __forceinline__ void sort_keys(u64 *sm, int t, int len, Sync &&sync) {
+    const int first = t * ITEMS, lenp = (len + ITEMS - 1) / ITEMS * ITEMS;
+    const bool on = first < len;
+    u64 k[ITEMS];
+    if (on) {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) k[i] = first + i < len ? sm[padded<ITEMS>(first + i)] : ~0ull;
+        batcher_sort(k);
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) sm[padded<ITEMS>(first + i)] = k[i];
+    }
+    sync();
+    for (int width = ITEMS; width < lenp; width <<= 1) {
+        const int a0 = first & ~(2 * width - 1), a1 = a0 + width, b1 = min(a0 + 2 * width, lenp);
+        const bool merge = on && a1 < b1;  // without a second run the keys stay
+        if (merge) {
+            const int diag = first - a0, lb = b1 - a1;
+            int lo = max(0, diag - lb), hi = min(diag, width);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (sm[padded<ITEMS>(a0 + mid)] < sm[padded<ITEMS>(a1 + diag - 1 - mid)]) lo = mid + 1;
+                else hi = mid;
+            }
+            int ai = a0 + lo, bi = a1 + diag - lo;
+            u64 ka = ai < a1 ? sm[padded<ITEMS>(ai)] : ~0ull, kb = bi < b1 ? sm[padded<ITEMS>(bi)] : ~0ull;
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) {
+                const bool take_a = ka < kb;
+                k[i] = take_a ? ka : kb;
+                const int idx = take_a ? ++ai : ++bi, end = take_a ? a1 : b1;
+                const u64 nk = idx < end ? sm[padded<ITEMS>(idx)] : ~0ull;
+                ka = take_a ? nk : ka;
+                kb = take_a ? kb : nk;
+            }
+        }
+        sync();
+        if (merge) {
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) sm[padded<ITEMS>(first + i)] = k[i];
+        }
+        sync();
+    }
+}
+
+// Sorts len <= THREADS x ITEMS keys with a group of THREADS threads: load(j) gives the j-th, store(at, key) takes
+// the one that belongs at position `at`. Depths spread over a tile's list, so the keys are dropped into as many buckets of equal depth
+// width (a monotone map) as there are keys, and each key then finds its place among the few of its bucket by
+// comparing with all of them: about 60 instructions a key where the merge sort takes 200. A list with more than
+// kBucketMost keys in a bucket (many equal depths, or a few far ones) is merge sorted.
+// keys: padded<ITEMS>(THREADS x ITEMS), cnt: THREADS x ITEMS, scratch: 3 per warp; `sync` is the group's barrier.
+constexpr uint32_t kBucketMost = 24;
+template <int ITEMS, class Sync>
+__device__ __noinline__ void sort_keys_apart(u64 *keys, int t, int len, Sync sync) {  // keeps its registers out of the callers
+    sort_keys<ITEMS>(keys, t, len, sync);
+}
+
+template <int THREADS, int ITEMS, class Sync, class Load, class Store>
+__device__ __forceinline__ void sort_spread(int len, u64 *keys, uint32_t *cnt, uint32_t *scratch, int t, Sync &&sync,
+                                            Load &&load, Store &&store) {
+    static_assert(THREADS * ITEMS <= 32768, "a bucket's start and count are packed into 32 bits");
+    constexpr int WARPS = THREADS / 32;
+    const int lane = t & 31, w = t >> 5;
+    u64 k[ITEMS];
+    uint32_t zlo = 0xffffffffu, zhi = 0u;  // depths are positive: their bits order as they do
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int j = t + i * THREADS;
+        if (j < len) {
+            k[i] = load(j);
+            zlo = min(zlo, (uint32_t)(k[i] >> 32));
+            zhi = max(zhi, (uint32_t)(k[i] >> 32));
+        }
+    }
+    int per = 1;  // buckets per thread
+    while (per * THREADS < len) per <<= 1;
+    const int nb = per * THREADS;
+    for (int b = t; b < nb; b += THREADS) cnt[b] = 0u;
+    zlo = __reduce_min_sync(0xffffffffu, zlo);
+    zhi = __reduce_max_sync(0xffffffffu, zhi);
+    if (WARPS > 1 && lane == 0) { scratch[w] = zlo; scratch[WARPS + w] = zhi; }
+    sync();
+    if (WARPS > 1) {
+        zlo = __reduce_min_sync(0xffffffffu, scratch[lane % WARPS]);
+        zhi = __reduce_max_sync(0xffffffffu, scratch[WARPS + lane % WARPS]);
+    }
+    const float z0 = __uint_as_float(zlo), width = __uint_as_float(zhi) - z0;
+    const float scale = width > 0.f ? (float)nb / width : 0.f;
+    auto bucket = [&](u64 key) {
+        return min((int)((__uint_as_float((uint32_t)(key >> 32)) - z0) * scale), nb - 1);
+    };
+    uint32_t rank[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (t + i * THREADS < len) rank[i] = atomicAdd(&cnt[bucket(k[i])], 1u);
+    sync();
+    // bucket starts: an exclusive scan, thread t taking buckets [t per, (t + 1) per)
+    uint32_t sum = 0, most = 0;
+    for (int q = 0; q < per; ++q) {
+        const uint32_t c = cnt[t * per + q];
+        sum += c;
+        most = max(most, c);
+    }
+    uint32_t incl = warp_incl_scan(sum);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (WARPS > 1) {
+        if (lane == 31) scratch[2 * WARPS + w] = incl;
+        if (lane == 0) scratch[w] = most;
+        sync();
+        most = __reduce_max_sync(0xffffffffu, scratch[lane % WARPS]);
+        const uint32_t before = lane < w ? scratch[2 * WARPS + lane] : 0u;  // WARPS <= 32
+        incl += __reduce_add_sync(0xffffffffu, before);
+    }
+    const bool spread = most <= kBucketMost;  // the same in all threads of the group
+    if (spread) {
+        uint32_t run = incl - sum;
+        for (int q = 0; q < per; ++q) {
+            const uint32_t c = cnt[t * per + q];
+            cnt[t * per + q] = run | (c << 16);  // starts below 2^15, counts at most kBucketMost
+            run += c;
+        }
+        sync();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (t + i * THREADS < len) keys[(cnt[bucket(k[i])] & 0xffffu) + rank[i]] = k[i];
+        sync();
+        for (int j = t; j < len; j += THREADS) {
+            const u64 key = keys[j];
+            const uint32_t sc = cnt[bucket(key)], first = sc & 0xffffu, n = sc >> 16;
+            uint32_t at = first;
+            for (uint32_t q = 0; q < n; ++q) at += keys[first + q] < key;
+            store((int)at, key);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (t + i * THREADS < len) keys[padded<ITEMS>(t + i * THREADS)] = k[i];
+        sync();
+        sort_keys_apart<ITEMS>(keys, t, len, sync);
+        for (int j = t; j < len; j += THREADS) store(j, keys[padded<ITEMS>(j)]);
+    }
+    sync();
+}
+
+// Sorts one segment (start, end, tile) of at most THREADS x ITEMS instances and writes its part of the lists.
+template <int THREADS, int ITEMS, class Sync>
+__device__ __forceinline__ void sort_segment(const BinArgs &a, uint4 rg, u64 *keys, uint32_t *cnt, uint32_t *scratch,
+                                             int t, Sync &&sync) {
+    sort_spread<THREADS, ITEMS>(
+        (int)(rg.y - rg.x), keys, cnt, scratch, t, sync, [&](int j) { return a.pairs[rg.x + j]; },
+        [&](int at, u64 key) {
+            a.inst_entry[rg.x + at] = (uint32_t)key;
+            a.inst_tile[rg.x + at] = rg.z;
+        });
+}
+
+// Lists of at most kCtaList entries: the longest by a whole CTA, those up to 1024 by 128 threads, those up to 256
+// by a warp. CTA b takes every gridDim-th of each class.
+constexpr int kListItems = 8, kListThreads = (int)kCtaList / kListItems;
+__global__ void __launch_bounds__(kListThreads, 2) k_sort_lists(const BinArgs a) {
+    extern __shared__ u64 sm[];
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(sm + padded<kListItems>(kCtaList));
+    __shared__ uint32_t scratch[3 * kListThreads / 32];
+    const int t = threadIdx.x, g = t >> 7, w = t >> 5;
+    const size_t T = (size_t)a.V.n_tiles * a.slabs;
+    const uint32_t n2 = a.aux->n_list[2], n1 = a.aux->n_list[1], n0 = a.aux->n_list[0];
+    for (uint32_t k = blockIdx.x; k < n2; k += gridDim.x)
+        sort_segment<kListThreads, kListItems>(a, a.lists[2 * T + k], sm, cnt, scratch, t, []() { __syncthreads(); });
+    for (uint32_t k = blockIdx.x * 4 + g; k < n1; k += gridDim.x * 4)
+        sort_segment<128, kListItems>(a, a.lists[T + k], sm + g * padded<kListItems>(1024), cnt + g * 1024, scratch + g * 12,
+                                   t & 127, [&]() { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); });
+    __syncthreads();
+    for (uint32_t k = blockIdx.x * 16 + w; k < n0; k += gridDim.x * 16)
+        sort_segment<32, kListItems>(a, a.lists[k], sm + w * padded<kListItems>(256), cnt + w * 256, scratch, t & 31,
+                                  []() { __syncwarp(); });
+}
+
+// Chunk q of the ceil(len / kBigList) chunks of a list [rg.x, rg.y).
+__device__ __forceinline__ uint2 chunk_of(uint4 job, uint32_t q) {
+    const uint64_t len = job.y - job.x, nch = (len + kBigList - 1) / kBigList;
+    return make_uint2(job.x + (uint32_t)(len * q / nch), job.x + (uint32_t)(len * (q + 1) / nch));
+}
+
+constexpr int kBigItems = (int)kBigList / 1024;
+
+// Lists of kCtaList to kBigList entries, and the chunks of longer ones (sorted in place).
+__global__ void __launch_bounds__(1024) k_sort_big(const BinArgs a) {
+    extern __shared__ u64 sm[];
+    __shared__ uint32_t scratch[3 * 32];
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(sm + padded<kBigItems>(kBigList));
+    const int t = threadIdx.x;
+    auto sync = []() { __syncthreads(); };
+    const uint32_t n3 = a.aux->n_list[3], nj = a.aux->n_jobs;
+    for (uint32_t k = blockIdx.x; k < n3; k += gridDim.x)
+        sort_segment<1024, kBigItems>(a, a.lists[3 * (size_t)a.V.n_tiles * a.slabs + k], sm, cnt, scratch, t, sync);
+    for (uint32_t k = blockIdx.x; k < nj; k += gridDim.x) {
+        const uint4 job = a.jobs[k];
+        const uint2 c = chunk_of(job, job.w);
+        // (every key is in a register or in shared memory before the first is stored)
+        sort_spread<1024, kBigItems>((int)(c.y - c.x), sm, cnt, scratch, t, sync,
+                                     [&](int j) { return a.pairs[c.x + j]; },
+                                     [&](int at, u64 key) { a.pairs[c.x + at] = key; });
+    }
+}
+
+// Number of keys of the sorted chunk c below p.
+__device__ __forceinline__ uint32_t keys_below(const u64 *pairs, uint2 c, u64 p) {
+    uint32_t lo = c.x, hi = c.y;
+    while (lo < hi) {
+        const uint32_t mid = lo + (hi - lo) / 2u;
+        if (pairs[mid] < p) lo = mid + 1u;
+        else hi = mid;
+    }
+    return lo - c.x;
+}
+
+// How many keys of each sorted chunk belong to the first target[0] and to the first target[1] keys of the whole list
+// (keys are unique): for each target the least p with that many keys below it, found 17-fold a round, one
+// candidate a warp, half of the warps a target: first among the multiples of 2^32 (the depths), then, where
+// several entries share the depth at the cut, among the keys.
+__device__ __forceinline__ void split_chunks(const BinArgs &a, uint4 job, uint32_t nch, const uint32_t (&target)[2],
+                                             uint32_t *from, uint32_t *to, uint32_t *s_below, uint32_t *s_range) {
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, half = w >> 4;
+    if (t == 0) { s_range[0] = 0xffffffffu; s_range[1] = 0u; }
+    __syncthreads();
+    for (uint32_t c = t; c < nch; c += 1024) {
+        const uint2 ch = chunk_of(job, c);
+        atomicMin(&s_range[0], (uint32_t)(a.pairs[ch.x] >> 32));
+        atomicMax(&s_range[1], (uint32_t)(a.pairs[ch.y - 1u] >> 32));
+    }
+    __syncthreads();
+    u64 lo[2], hi[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) { lo[h] = s_range[0]; hi[h] = (u64)s_range[1] + 1u; }
+#pragma unroll
+    for (int shift = 32; shift >= 0; shift -= 32) {
+        while (lo[0] < hi[0] || lo[1] < hi[1]) {  // uniform for the CTA
+            auto pivot = [&](int h, int k) {
+                const u64 span = hi[h] - lo[h], q = span / 17u;
+                return q ? lo[h] + q * (u64)(k + 1) : lo[h] + min((u64)k, span);
+            };
+            const u64 p = pivot(half, w & 15) << shift;
+            uint32_t below = 0;
+            for (uint32_t c = lane; c < nch; c += 32) below += keys_below(a.pairs, chunk_of(job, c), p);
+            below = __reduce_add_sync(0xffffffffu, below);
+            if (lane == 0) s_below[w] = below;
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                int k = 0;
+                while (k < 16 && s_below[16 * h + k] < target[h]) ++k;
+                const u64 nlo = k > 0 ? min(pivot(h, k - 1) + 1u, hi[h]) : lo[h], nhi = k < 16 ? pivot(h, k) : hi[h];
+                lo[h] = nlo;
+                hi[h] = nhi;
+            }
+            __syncthreads();
+        }
+        if (shift == 32) {  // the cut lies in (lo - 1, lo] << 32
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                hi[h] = lo[h] << 32;
+                lo[h] = (lo[h] > 0 ? lo[h] - 1u : 0u) << 32;
+            }
+            // most cuts fall between two depths: then the search among the keys has nothing to do
+            uint32_t below = 0;
+            for (uint32_t c = lane; c < nch; c += 32) below += keys_below(a.pairs, chunk_of(job, c), hi[half]);
+            below = __reduce_add_sync(0xffffffffu, below);
+            if (lane == 0) s_below[w] = below;
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (s_below[16 * h] == target[h]) lo[h] = hi[h];
+            __syncthreads();
+        }
+    }
+    for (uint32_t c = t; c < nch; c += 1024) {
+        const uint2 ch = chunk_of(job, c);
+        from[c] = keys_below(a.pairs, ch, lo[0]);
+        to[c] = keys_below(a.pairs, ch, lo[1]);
+    }
+    __syncthreads();
+}
+
+// The lists of more than kBigList entries, from their sorted chunks: job q produces the q-th of as many parts of
+// the whole list, gathering its keys from all chunks and sorting them once more.
+__global__ void __launch_bounds__(1024) k_merge_chunks(const BinArgs a, uint32_t max_chunks) {
+    extern __shared__ u64 sm[];
+    __shared__ uint32_t s_warp[33], s_below[32], s_range[2], scratch[3 * 32];
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(sm + padded<kBigItems>(kBigList));
+    uint32_t *from = cnt, *to = from + max_chunks;  // needed before the sort only (max_chunks <= kBigList / 2)
+    const int t = threadIdx.x;
+    const uint32_t nj = a.aux->n_jobs;
+    for (uint32_t k = blockIdx.x; k < nj; k += gridDim.x) {
+        const uint4 job = a.jobs[k];
+        const uint32_t nch = (job.y - job.x + kBigList - 1u) / kBigList;
+        const uint2 part = chunk_of(job, job.w);
+        const uint32_t target[2] = {part.x - job.x, part.y - job.x};
+        split_chunks(a, job, nch, target, from, to, s_below, s_range);
+        uint32_t run = 0;
+        for (uint32_t c0 = 0; c0 < nch; c0 += 1024) {  // a chunk a thread finds its place, then the CTA copies them
+            const uint32_t c = c0 + t, n = c < nch ? to[c] - from[c] : 0u;
+            uint32_t tot;
+            const uint32_t at = run + block_excl_scan(n, s_warp, tot);
+            run += tot;
+            if (c < nch) to[c] = at;  // from now on: the part's offset of this chunk's keys
+        }
+        __syncthreads();
+        const int len = (int)(part.y - part.x), lane = t & 31;
+        for (uint32_t c = t >> 5; c < nch; c += 32) {
+            const uint32_t at = to[c], n = (c + 1 < nch ? to[c + 1] : (uint32_t)len) - at;
+            const uint32_t src = chunk_of(job, c).x + from[c];
+            for (uint32_t j = lane; j < n; j += 32) sm[padded<kBigItems>((int)(at + j))] = a.pairs[src + j];
+        }
+        __syncthreads();
+        sort_spread<1024, kBigItems>(len, sm, cnt, scratch, t, []() { __syncthreads(); },
+                                     [&](int j) { return sm[padded<kBigItems>(j)]; },
+                                     [&](int at, u64 key) {
+                                         a.inst_entry[part.x + at] = (uint32_t)key;
+                                         a.inst_tile[part.x + at] = job.z;
+                                     });
+    }
+}
+
+static int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
+
+template <bool EMIT, bool SHARED, bool SLABS>
+static cudaError_t launch_instances_t(const BinArgs &a, uint32_t grid, uint32_t threads, int smem, cudaStream_t s) {
+    if (smem) {  // on every call: the attribute belongs to the current device
+        const cudaError_t e = cudaFuncSetAttribute(k_instances<EMIT, SHARED, SLABS>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_instances<EMIT, SHARED, SLABS><<<grid, threads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <bool EMIT>
+static cudaError_t launch_instances(const BinArgs &a, bool shared, uint32_t grid, uint32_t threads, int smem,
+                                    cudaStream_t s) {
+    if (a.slabs > 1)
+        return shared ? launch_instances_t<EMIT, true, true>(a, grid, threads, smem, s)
+                      : launch_instances_t<EMIT, false, true>(a, grid, threads, smem, s);
+    return shared ? launch_instances_t<EMIT, true, false>(a, grid, threads, smem, s)
+                  : launch_instances_t<EMIT, false, false>(a, grid, threads, smem, s);
 }
 
 cudaError_t launch_bin(const BinArgs &a, cudaStream_t s) {
-    cudaError_t e;
-    const uint32_t nE = a.n_entries;
-    if (nE == 0) {  // no splats: every tile is empty
-        e = cudaMemsetAsync(a.ranges, 0, sizeof(uint2) * (size_t)a.V.n_tiles, s);
-        if (e != cudaSuccess) return e;
-        if (a.build_queue) k_lpt_queue<<<1, 1024, 0, s>>>(a.ranges, (uint32_t)a.V.n_tiles, a.queue);
-        return cudaGetLastError();
-    }
-    // 1. depth sort of all entries; key = z32 bits (culled: 0xffffffff), value = entry
-    k_depth_keys<<<ceil_div_u64(nE, 256), 256, 0, s>>>(a.binrec, a.dkey[0], nE);
-    uint32_t *dk[2] = {a.dkey[0], a.dkey[1]}, *dv[2] = {a.dval[0], a.dval[1]};
-    e = radix_sort(dk, dv, true, nullptr, nE, 32, a.hist, a.partials, s);
+    const uint32_t n_tiles = (uint32_t)a.V.n_tiles;
+    cudaError_t e = cudaMemsetAsync(a.aux, 0, sizeof(TileAux) + sizeof(uint32_t) * (size_t)n_tiles * a.slabs, s);
     if (e != cudaSuccess) return e;
-    const uint32_t *sorted_e = dv[0];  // 4 passes: result back in buffer 0
-    // 2. tiles touched in depth order -> exclusive scan -> emission offsets
-    k_gather_counts<<<ceil_div_u64(nE, 128), 128, 0, s>>>(sorted_e, a.binrec, a.rcount, a.rinfo, nE, a.n, a.V);
-    e = exclusive_scan(a.rcount, a.rcount, nE, a.partials, nullptr, s);
-    if (e != cudaSuccess) return e;
-    k_set_count<<<1, 1, 0, s>>>(a.total, a.cap, a.header);
-    // 3. emit (tile, entry) instances in depth order
-    EmitArgs ea;
-    ea.n_entries = nE; ea.n = a.n; ea.rinfo = a.rinfo; ea.offsets = a.rcount; ea.rec = a.rec;
-    ea.binrec = a.binrec; ea.total = a.total; ea.ikey = a.ikey[0]; ea.ival = a.ival[0]; ea.cap = a.cap;
-    ea.err = a.err; ea.V = a.V;
-    k_emit<<<ceil_div_u64(nE, 128), 128, 0, s>>>(ea);
-    // 4. stable sort by global tile id keeps the depth order inside each tile
-    uint32_t *ik[2] = {a.ikey[0], a.ikey[1]}, *iv[2] = {a.ival[0], a.ival[1]};
-    const uint32_t cap32 = (uint32_t)a.cap;
-    if (a.tile_bits > 0 && a.cap > 0) {
-        e = radix_sort(ik, iv, false, a.header, cap32, a.tile_bits, a.hist, a.partials, s);
+    const int sms = sm_count();
+    // 1. instances per tile: counted in shared memory while a view's counters fit; a CTA takes as many entries as
+    // still leave a few CTAs for every SM
+    BinArgs c = a;
+    const uint32_t counters = most_tiles(a.V) * a.slabs;
+    const bool shared = inst_shared(a.n, a.V);  // as the layout was made for
+    c.per_cta = inst_entries(a.n, a.n_views);
+    c.parts = inst_parts(a.n, a.n_views);
+    const uint32_t grid = ceil_div_u64((uint64_t)a.n, c.per_cta) * c.parts * (uint32_t)a.n_views;
+    const uint32_t threads = min(c.per_cta, (uint32_t)kInstThreads);
+    const int inst_smem = shared ? (int)(sizeof(uint32_t) * counters) : 0;
+    if (a.n > 0) {
+        if (a.slabs > 1) k_depth_range<<<dim3(ceil_div_u64((uint64_t)a.n, 2048), (uint32_t)a.n_views), 256, 0, s>>>(a);
+        e = launch_instances<false>(c, shared, grid, threads, inst_smem, s);
         if (e != cudaSuccess) return e;
     }
-    const int res = ((a.tile_bits + 7) / 8) & 1;
-    // 5. tile ranges
-    e = cudaMemsetAsync(a.ranges, 0, sizeof(uint2) * (size_t)a.V.n_tiles, s);
+    // 2. segments, ranges, sort classes, queue
+    const uint32_t per = 1024u * ceil_div_u64(n_tiles, 1024ull * kTileBlocks);
+    const uint32_t nblk = ceil_div_u64(n_tiles, per);
+    k_tile_sums<<<nblk, 1024, 0, s>>>(a, per);
+    k_tile_index<<<nblk, 1024, 0, s>>>(a, per);
+    if (a.n == 0) return cudaGetLastError();
+    // 3. append
+    e = launch_instances<true>(c, shared, grid, threads, inst_smem, s);
     if (e != cudaSuccess) return e;
-    if (a.cap > 0) k_tile_ranges<<<ceil_div_u64(ceil_div_u64(a.cap, 4), 256), 256, 0, s>>>(ik[res], a.header, a.ranges, (uint32_t)a.V.n_tiles);
-    // 6. longest-first queue for the persistent render
-    if (a.build_queue) k_lpt_queue<<<1, 1024, 0, s>>>(a.ranges, (uint32_t)a.V.n_tiles, a.queue);
+    // 4. sort: a tile's list has at most one entry per splat
+    constexpr int list_smem = (int)(sizeof(u64) * padded<kListItems>(kCtaList) + sizeof(uint32_t) * kCtaList);
+    e = cudaFuncSetAttribute(k_sort_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, list_smem);
+    if (e != cudaSuccess) return e;
+    k_sort_lists<<<(uint32_t)min((uint64_t)(2 * sms), (uint64_t)n_tiles * a.slabs), kListThreads, list_smem, s>>>(a);
+    const uint64_t longest = (uint64_t)a.n < a.cap ? (uint64_t)a.n : a.cap;
+    if (longest > kCtaList) {
+        constexpr int smem = (int)(sizeof(u64) * padded<kBigItems>(kBigList) + sizeof(uint32_t) * kBigList);
+        e = cudaFuncSetAttribute(k_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        k_sort_big<<<sms, 1024, smem, s>>>(a);
+    }
+    if (longest > kBigList) {
+        const uint32_t max_chunks = ceil_div_u64(longest, kBigList);  // at most 4096: 67,108,864 entries in all
+        constexpr int smem = (int)(sizeof(u64) * padded<kBigItems>(kBigList) + sizeof(uint32_t) * kBigList);
+        e = cudaFuncSetAttribute(k_merge_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        k_merge_chunks<<<sms, 1024, smem, s>>>(a, max_chunks);
+    }
     return cudaGetLastError();
 }
 

@@ -109,46 +109,109 @@ constexpr int kScanMaxPartials = 1024 * 16;
 
 inline uint32_t ceil_div_u64(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
-// bins: [header 256][dkey 2 x nV][dval 2 x nV][rank counts nV][rank info nV x 16][ikey 2 x cap]
-//       [ival 2 x cap][ranges T x 8][queue T][hist 256 x nblk][partials]
-// header: u32 n_inst (instances actually listed) at 0, u32 queue counters at 4 and 8, u64 count of
-// the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval).
-struct BinsLayout {
-    uint64_t dkey[2], dval[2], rcount, rinfo, ikey[2], ival[2], ranges, queue, hist, partials, bytes;
-    uint32_t n_tiles;
-    uint32_t nblk_entries, nblk_inst;  // radix CTAs for the depth sort and the tile sort
-    int tile_passes;                   // 8-bit passes of the tile sort
-};
-
 inline int bits_for(uint32_t v) {  // bits needed to hold values 0..v-1
     int b = 0;
     while (b < 32 && (1ull << b) < (uint64_t)v) ++b;
     return b;
 }
 
-inline BinsLayout bins_layout(int32_t n, int32_t n_views, uint32_t n_tiles, uint64_t cap) {
-    const uint64_t nv = (uint64_t)n * (uint64_t)n_views;
+// Tile lists are sorted by CTAs: up to kCtaList entries by one CTA of 512 threads (or a part of one), up to
+// kBigList by one CTA of 1024, longer ones in chunks of at most kBigList.
+constexpr uint32_t kCtaList = 4096, kBigList = 16384;
+constexpr int kLptBuckets = 128;   // list-length buckets of the longest-first queue
+constexpr int kListClasses = 4;    // <= 256, <= 1024, <= kCtaList, <= kBigList entries
+constexpr uint32_t kTileBlocks = 512;  // most CTAs of the tile-index kernels
+
+// Counters of the tile index, cleared by every ges_bin together with the tile counts after them.
+struct TileAux {
+    uint32_t partial[kTileBlocks];     // instances of each CTA's tiles
+    uint32_t bucket[kLptBuckets];      // tiles per list-length bucket
+    uint32_t bucket_cur[kLptBuckets];  // queue slots taken per bucket
+    uint32_t n_list[kListClasses];     // segments per sort class
+    uint32_t n_jobs;                   // chunks of longer ones
+    uint32_t depth_hi[kMaxViews], depth_lo_inv[kMaxViews];  // greatest depth bits of a view's entries, and of ~bits
+};
+
+// bins: [header 256][instance tile cap x 4][instance entry cap x 4][unsorted instances cap x 8][ranges T x 8]
+//       [queue T][TileAux, counts of the G = T x slabs segments x 4][class lists 4 x G x 16][chunk jobs x 16]
+//       [places: CTAs per view x G x 4]
+// header: u32 n_inst (instances actually listed) at 0, u32 queue counters at 4 and 8, u64 count of
+// the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval).
+struct BinsLayout {
+    uint64_t tile, entry, pairs, ranges, queue, aux, counts, lists, jobs, places, bytes;
+    uint32_t n_tiles;
+};
+
+// The instance kernels: CTAs of up to kInstThreads, each with consecutive entries of one view.
+constexpr int kInstThreads = 512;
+constexpr uint32_t kSharedCounters = 24576;  // most counters in shared memory (96 KB: two CTAs per SM)
+constexpr uint32_t kMostSlabs = 64;
+
+// Entries per CTA: more share a tile's atomic and write its instances side by side, up to 8 rounds of
+// the CTA (at 16 and 32 the open segments of all CTAs outgrow L2: binning of 8 views of 1.5M splats 1.23 ms
+// at 8, 1.25 at 4, 1.32 at 16, 1.59 at 32), and no more than leaves some 600 CTAs; at least 64.
+inline uint32_t inst_entries(int32_t n, int32_t n_views) {
+    const uint64_t each = (uint64_t)n * (uint64_t)n_views / 608u;
+    if (each >= (uint64_t)kInstThreads) return (uint32_t)kInstThreads * (uint32_t)(each / kInstThreads > 8 ? 8 : each / kInstThreads);
+    return each < 64u ? 64u : (uint32_t)((each + 31u) / 32u * 32u);
+}
+
+// CTAs that share the rounds of the same entries, where there are few entries.
+inline uint32_t inst_parts(int32_t n, int32_t n_views) {
+    const uint64_t warps = ((uint64_t)n * (uint64_t)n_views + 31u) / 32u;
+    const uint64_t parts = warps ? 8u * 608u / warps : 1u;
+    return parts < 1u ? 1u : parts > 8u ? 8u : (uint32_t)parts;
+}
+
+inline uint32_t most_tiles(const ViewSet &V) {  // of any view
+    uint32_t most = 0;
+    for (int v = 0; v < V.n_views; ++v) {
+        const uint32_t t = (uint32_t)(V.tile_base[v + 1] - V.tile_base[v]);
+        if (t > most) most = t;
+    }
+    return most;
+}
+
+// Depth slabs per tile (a power of two). Where the entries are many for the tiles, lists would be too long for a
+// CTA's shared memory; a tile's segment is then split into slabs of equal depth width over its view's depths,
+// which are counted, filled and sorted as segments of their own. Measured, binning without and with slabs: 564k
+// splats in a 283x268 view, 1,844 entries a tile, 233 and 170 us; 278k in 119x100, 5,352 a tile, 238 and 90 us;
+// below 512 the lists that are too long are few, and the extra pass over the depths costs more.
+inline uint32_t depth_slabs(int32_t n, const ViewSet &V) {
+    const uint64_t density = V.n_tiles > 0 ? (uint64_t)n * (uint64_t)V.n_views / (uint64_t)V.n_tiles : 0;
+    uint32_t s = 1;
+    if (density >= 512u)
+        while (s < kMostSlabs && (uint64_t)s * 32u < density && most_tiles(V) * 2u * s <= kSharedCounters) s *= 2;
+    return s;
+}
+
+// Whether a CTA counts its entries' instances in shared memory: its counters are cleared and read once a CTA, which
+// its entries have to pay for.
+inline bool inst_shared(int32_t n, const ViewSet &V) {
+    const uint32_t counters = most_tiles(V) * depth_slabs(n, V);
+    return counters <= kSharedCounters && counters <= 16u * inst_entries(n, V.n_views);
+}
+
+inline BinsLayout bins_layout(int32_t n, const ViewSet &V, uint64_t cap) {
+    const uint32_t n_tiles = (uint32_t)V.n_tiles;
+    const uint64_t n_segs = (uint64_t)n_tiles * depth_slabs(n, V);
     BinsLayout L;
     L.n_tiles = n_tiles;
     uint64_t off = 256;
-    for (int i = 0; i < 2; ++i) { L.dkey[i] = off; off = align256(off + nv * 4); }
-    for (int i = 0; i < 2; ++i) { L.dval[i] = off; off = align256(off + nv * 4); }
-    L.rcount = off; off = align256(off + nv * 4 + 4);
-    L.rinfo = off; off = align256(off + nv * 16);
-    for (int i = 0; i < 2; ++i) { L.ikey[i] = off; off = align256(off + cap * 4); }
-    for (int i = 0; i < 2; ++i) { L.ival[i] = off; off = align256(off + cap * 4); }
+    L.tile = off; off = align256(off + cap * 4);
+    L.entry = off; off = align256(off + cap * 4);
+    L.pairs = off; off = align256(off + cap * 8);
     L.ranges = off; off = align256(off + (uint64_t)n_tiles * 8);
     L.queue = off; off = align256(off + (uint64_t)n_tiles * 4);
-    L.nblk_entries = ceil_div_u64(nv > 0 ? nv : 1, kSortTile);
-    L.nblk_inst = ceil_div_u64(cap > 0 ? cap : 1, kSortTile);
-    uint32_t nblk = L.nblk_entries > L.nblk_inst ? L.nblk_entries : L.nblk_inst;
-    L.hist = off; off = align256(off + (uint64_t)256 * nblk * 4);
-    uint64_t scan_n = (uint64_t)256 * nblk;
-    if (nv > scan_n) scan_n = nv;
-    L.partials = off; off = align256(off + ((uint64_t)ceil_div_u64(scan_n, kScanTile) + 1) * 4);
+    L.aux = off; L.counts = off + sizeof(TileAux); off = align256(L.counts + n_segs * 4);
+    L.lists = off; off = align256(off + n_segs * 16 * kListClasses);
+    // a list of more than kBigList entries has ceil(len / kBigList) < 2 len / kBigList chunks
+    L.jobs = off; off = align256(off + (cap / (kBigList / 32) + 2) * 16);
+    L.places = off;
+    if (inst_shared(n, V))
+        off = align256(off + 4ull * n_segs * ceil_div_u64(n > 0 ? (uint64_t)n : 1, inst_entries(n, V.n_views)) *
+                                 inst_parts(n, V.n_views));
     L.bytes = off;
-    int tb = bits_for(n_tiles);
-    L.tile_passes = tb == 0 ? 0 : (tb + 7) / 8;
     return L;
 }
 
@@ -434,36 +497,26 @@ struct PreBwdArgs {
     ViewSet V;
 };
 
-struct EmitArgs {
-    uint32_t n_entries;
-    int n;  // splats per view
-    const uint4 *rinfo;        // per rank: entry, hit mask, key of the box's first tile, box width | tiles_x << 6
-    const uint32_t *offsets;   // exclusive scan of tiles touched in that order
+struct BinArgs {
+    int n, n_views;
     const float4 *rec;
     const uint4 *binrec;
     const unsigned long long *total;  // instances found by the preprocess
-    uint32_t *ikey, *ival;
-    uint64_t cap;
-    uint32_t *err;
-    ViewSet V;
-};
-
-struct BinArgs {
-    int n, n_views;
-    uint32_t n_entries;
-    const float4 *rec;
-    const uint4 *binrec;
-    const unsigned long long *total;
     uint32_t *err;
     // bins
     uint32_t *header;  // [0] n_inst
-    uint32_t *dkey[2], *dval[2], *rcount, *ikey[2], *ival[2];
-    uint4 *rinfo;
+    uint32_t *inst_tile, *inst_entry;
+    unsigned long long *pairs;  // depth bits << 32 | entry, grouped by tile
     uint2 *ranges;
     uint32_t *queue;
-    uint32_t *hist, *partials;
+    TileAux *aux;
+    uint32_t *counts;  // instances per segment (tile x slabs + slab), then the next free slot of it
+    uint4 *lists;      // [kListClasses][segments]: start, end, tile, -
+    uint4 *jobs;       // start, end, tile, chunk
+    uint32_t *places;  // [CTAs of the instance kernels per view][segments]: where a CTA's instances of one start
+    uint32_t slabs;
     uint64_t cap;
-    int tile_bits;
+    uint32_t per_cta, parts;  // entries a CTA of the instance kernels takes, CTAs that share them
     bool build_queue;
     ViewSet V;
 };

@@ -15,6 +15,7 @@
 // centres never reach; tens of thousands of coincident centres would) takes the best of the first
 // 65,536 in ring order instead, so no input makes the search quadratic.
 #include "ges_internal.cuh"
+#include "sort_net.cuh"
 
 namespace ges {
 
@@ -413,7 +414,7 @@ __device__ __forceinline__ void add_found(Found &f, float d, uint32_t id) {
     if (db < w.x || (db == w.x && id < w.y)) f.col[worst * f.stride] = make_uint2(db, id);
 }
 
-// The column sorted by (distance, index), as indices; missing entries -1. Batcher's odd-even merge sort.
+// The column sorted by (distance, index), as indices; missing entries -1.
 __device__ __forceinline__ void sorted_indices(const Found &f, int32_t (&out)[kK]) {
     unsigned long long key[kK];
 #pragma unroll
@@ -421,20 +422,7 @@ __device__ __forceinline__ void sorted_indices(const Found &f, int32_t (&out)[kK
         const uint2 c = f.col[k * f.stride];
         key[k] = k < f.n ? ((unsigned long long)c.x << 32) | c.y : ~0ull;
     }
-#pragma unroll
-    for (int p = 1; p < kK; p <<= 1)
-#pragma unroll
-        for (int q = p; q >= 1; q >>= 1)
-#pragma unroll
-            for (int j = q % p; j + q < kK; j += 2 * q)
-#pragma unroll
-                for (int i = 0; i < q; ++i)
-                    if (i + j + q < kK && (i + j) / (2 * p) == (i + j + q) / (2 * p)) {
-                        const unsigned long long lo = key[i + j], hi = key[i + j + q];
-                        const bool swap = hi < lo;
-                        key[i + j] = swap ? hi : lo;
-                        key[i + j + q] = swap ? lo : hi;
-                    }
+    batcher_sort(key);
 #pragma unroll
     for (int k = 0; k < kK; ++k) out[k] = (int32_t)(uint32_t)key[k];
 }

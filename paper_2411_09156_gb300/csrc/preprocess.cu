@@ -81,7 +81,7 @@ __device__ __forceinline__ void warp_tile_tests(const TileJob &J, int lane, int 
                                                 uint4 *jobs, uint32_t &tiles, uint32_t &mask) {
     tiles = 0;
     mask = 0;
-    warp_tile_rounds(J, lane, lw, lh, tw, th, jobs,
+    warp_tile_rounds(J, lane, lw, lh, tw, th, jobs, 0u, 1u,
                      [&](uint32_t hits, uint32_t lo, uint32_t len, uint32_t first, int, int, uint32_t, bool) {
                          if (!len) return;
                          const uint32_t bits = (hits >> lo) & (len == 32u ? 0xffffffffu : ((1u << len) - 1u));

@@ -30,9 +30,10 @@ constexpr int kJobWords = 3;
 // jobs: the warp's table (kJobWords * 32 uint4 of shared memory): each lane publishes its
 // ellipse, pixel box, first test index and a multiplier for dividing by its box width once,
 // and each round reads its owner's from there.
+// Only every `parts`-th round from round `part` on is run (the other parts by other warps).
 template <class OnRound>
 __device__ __forceinline__ void warp_tile_rounds(const TileJob &J, int lane, int lw, int lh, int tw, int th,
-                                                 uint4 *jobs, OnRound &&on_round) {
+                                                 uint4 *jobs, uint32_t part, uint32_t parts, OnRound &&on_round) {
     constexpr uint32_t FULL = 0xffffffffu;
     uint32_t incl = J.nbox;
 #pragma unroll
@@ -56,7 +57,7 @@ __device__ __forceinline__ void warp_tile_rounds(const TileJob &J, int lane, int
         jobs[kJobWords * lane + 2] = make_uint4(J.xs, J.ys, excl, m);
         __syncwarp();
     }
-    for (uint32_t j0 = 0; j0 < wtotal; j0 += 32) {
+    for (uint32_t j0 = 32u * part; j0 < wtotal; j0 += 32u * parts) {
         const uint32_t j = j0 + (uint32_t)lane;
         int owner = 0;
 #pragma unroll
