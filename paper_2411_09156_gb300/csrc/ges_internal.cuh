@@ -326,16 +326,17 @@ __device__ __forceinline__ void pixel_box(float u, float v, float ext_x, float e
     x0 = (int)fx0; x1 = (int)fx1; y0 = (int)fy0; y1 = (int)fy1;
 }
 
-// Screen-space evaluation of one (pixel, splat) pair, shared by forward and
-// backward so that both take bit-identical decisions.
+// Screen-space evaluation of one (pixel, splat) pair, shared by forward and backward so that both take
+// bit-identical decisions: the pair blends if Q <= q_cut and alpha >= alpha_min. (Where a lane outside the support
+// evaluates alpha all the same, p may be +inf and G, alpha 0; Q is finite or +inf, never NaN.)
 struct PairEval {
-    float Q, lq, p, G, alpha_raw, alpha;  // lq = log2 Q
+    float lq, p, G, alpha_raw, alpha;  // lq = log2 Q
 };
 
-// Q = d^T C d of the pair (clamped at 0), d = (dx, dy), C the conic [a, b2/2; b2/2, c].
-__device__ __forceinline__ float pair_q(float dx, float dy, float a, float b2, float c) {
-    const float t = __fmaf_rn(a, dx, __fmul_rn(b2, dy));
-    return fmaxf(__fmaf_rn(__fmul_rn(c, dy), dy, __fmul_rn(dx, t)), 0.f);
+// Q = d^T C d of the pair (clamped at 0), d = (dx, dy), C the conic [a, b2/2; b2/2, c], from the products b2 dy and
+// c dy.
+__device__ __forceinline__ float pair_q(float dx, float dy, float a, float b2dy, float cdy) {
+    return fmaxf(__fmaf_rn(cdy, dy, __fmul_rn(dx, __fmaf_rn(a, dx, b2dy))), 0.f);
 }
 
 // p = Q^(beta/2) (Q = 0 gives 0), G = exp(-p/2), alpha = min(alpha_max, o G).
@@ -344,29 +345,7 @@ __device__ __forceinline__ void pair_alpha(float Q, float hb, float o, float alp
     const float p = ex2_approx(__fmul_rn(hb, lq));
     const float G = ex2_approx(__fmul_rn(kNegHalfLog2e, p));
     const float ar = __fmul_rn(o, G);
-    r.Q = Q; r.lq = lq; r.p = p; r.G = G; r.alpha_raw = ar; r.alpha = fminf(alpha_max, ar);
-}
-
-// Returns false if the pair is outside the support (Q > q_cut) or alpha < alpha_min. A lane
-// outside the support skips the special-function work (r then holds Q only).
-__device__ __forceinline__ bool eval_pair(float dx, float dy, float a, float b2, float c, float qcut, float hb,
-                                          float o, float alpha_max, float alpha_min, PairEval &r) {
-    const float Q = pair_q(dx, dy, a, b2, c);
-    r.Q = Q;
-    if (Q > qcut) return false;
-    pair_alpha(Q, hb, o, alpha_max, r);
-    return r.alpha >= alpha_min;
-}
-
-// The same decision and values without a branch: every lane does the special-function work and
-// r is filled in full (outside the support p may be +inf and G, alpha 0; Q is finite or +inf,
-// never NaN). For a loop whose body runs on every lane of the warp anyway, where the branch
-// only adds divergence and reconvergence work.
-__device__ __forceinline__ bool eval_pair_all(float dx, float dy, float a, float b2, float c, float qcut, float hb,
-                                              float o, float alpha_max, float alpha_min, PairEval &r) {
-    const float Q = pair_q(dx, dy, a, b2, c);
-    pair_alpha(Q, hb, o, alpha_max, r);
-    return Q <= qcut && r.alpha >= alpha_min;
+    r.lq = lq; r.p = p; r.G = G; r.alpha_raw = ar; r.alpha = fminf(alpha_max, ar);
 }
 
 // Real spherical harmonics up to degree 3 (Condon-Shortley phase, l-major,

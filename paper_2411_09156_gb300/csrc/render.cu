@@ -261,8 +261,7 @@ __global__ void __launch_bounds__(TW *TH, 9 * 128 / (TW * TH)) k_render_fwd(cons
                 float dx, dy, b2dy, cdy;
                 unpack2(d, dx, dy);
                 unpack2(mul2(s0.y, pack2(dy, dy)), b2dy, cdy);
-                // Q as pair_q forms it
-                const float Q = fmaxf(__fmaf_rn(cdy, dy, __fmul_rn(dx, __fmaf_rn(r1.x, dx, b2dy))), 0.f);
+                const float Q = pair_q(dx, dy, r1.x, b2dy, cdy);
                 if (Q > r1.y) continue;
                 PairEval pe;
                 pair_alpha(Q, r1.z, r1.w, a.alpha_max, pe);
@@ -332,20 +331,11 @@ __device__ __forceinline__ void halve(float *g, int lane) {
     }
 }
 
-template <int NV>
-__device__ __forceinline__ float warp_reduce_n(float (&g)[NV], int lane) {
-    static_assert(NV >= 9 && NV <= 16, "four halvings leave one value");
-    constexpr int N1 = (NV + 1) / 2, N2 = (N1 + 1) / 2, N3 = (N2 + 1) / 2;
-    halve<16, NV>(g, lane);
-    halve<8, N1>(g, lane);
-    halve<4, N2>(g, lane);
-    halve<2, N3>(g, lane);
-    return g[0] + __shfl_xor_sync(0xffffffffu, g[0], 1);
-}
-
-// warp_reduce_n<NV> with the level at offset 16 given as the values each lane keeps and sends
-// (NV even): keep[i] and send[i] are positions i and i + NV/2 in the order of the lane's half.
-template <int NV>
+// The same with the level at offset 16 given as the values each lane keeps and sends (NV even): keep[i] and
+// send[i] are positions i and i + NV/2 in the order of the lane's half. Selections are left out at offset 8:
+// with EXCHANGED position 0 and its partner there come already exchanged in the lanes with bit 8 set, and a value
+// without a partner is summed by both lanes (the one whose label is -1 is not written).
+template <int NV, bool EXCHANGED>
 __device__ __forceinline__ float warp_reduce_split(const float (&keep)[NV / 2], const float (&send)[NV / 2],
                                                    int lane) {
     static_assert(NV % 2 == 0 && NV >= 10 && NV <= 16, "three halvings after the split leave one value");
@@ -353,13 +343,24 @@ __device__ __forceinline__ float warp_reduce_split(const float (&keep)[NV / 2], 
     float g[N1];
 #pragma unroll
     for (int i = 0; i < N1; ++i) g[i] = keep[i] + __shfl_xor_sync(0xffffffffu, send[i], 16);
-    halve<8, N1>(g, lane);
+    const bool up = lane & 8;
+#pragma unroll
+    for (int i = 0; i < N2; ++i) {
+        if (EXCHANGED && i == 0) {
+            g[0] = g[0] + __shfl_xor_sync(0xffffffffu, g[N2], 8);
+        } else if (N2 + i < N1) {
+            const float sd = up ? g[i] : g[N2 + i], kp = up ? g[N2 + i] : g[i];
+            g[i] = kp + __shfl_xor_sync(0xffffffffu, sd, 8);
+        } else {
+            g[i] = g[i] + __shfl_xor_sync(0xffffffffu, g[i], 8);
+        }
+    }
     halve<4, N2>(g, lane);
     halve<2, N3>(g, lane);
     return g[0] + __shfl_xor_sync(0xffffffffu, g[0], 1);
 }
 
-// The value index that lane's pair holds after warp_reduce_n<NV>, or -1 (a padding zero).
+// The value index that lane's pair holds after the reduction, or -1 (no value).
 __device__ __forceinline__ int reduce_label(int nv, int lane) {
     int start = 0, valid = nv, n = nv;
     for (int d = 16; d >= 2; d >>= 1) {
@@ -386,19 +387,20 @@ __global__ void __launch_bounds__(TW *TH) k_render_bwd(const BwdArgs a) {
     // The gradient values a pair contributes, in reduction order: the level at lane offset 16 pairs
     // position i with i + NV/2, and the pairs are chosen so that few of them need a per-event swap
     // (see the event body):
-    //   FULL:   mean.x  S.xx  S.xy     red    green  blue   beta  |  mean.y  S.yy  opacity  n.x  n.y  n.z  depth
-    //   colour: mean.x  S.xx  S.xy     red    blue                |  mean.y  S.yy  opacity  green  beta
+    //   FULL:   red    mean.x  S.xx  S.xy     green  blue  beta  |  n.x    mean.y  S.yy  opacity  n.y  n.z  depth
+    //   colour: mean.x  S.xx  S.xy     red    blue               |  mean.y  S.yy  opacity  green  beta
     // (S = Sigma'). Position p goes to slot (kSlots >> 4p) & 15 of the splat's 16-float
     // accumulator: 0-1 mean, 2-4 Sigma' xx xy yy, 5 opacity, 6 beta, 7 depth, 8-10 colour,
     // 12-14 normal (slots 11 and 15, and without FULL 7 and 12-14, stay 0). After the reduction
     // this lane's pair holds position `lab`.
     constexpr int NV = FULL ? 14 : 10;
     constexpr int H1 = NV / 2;
-    constexpr unsigned long long kSlots = FULL ? 0x7EDC5416A98320ull : 0x69541A8320ull;
+    constexpr unsigned long long kSlots = FULL ? 0x7ED541C6A93208ull : 0x69541A8320ull;
     const int lab = reduce_label(NV, lane);
     const int gslot = lab < 0 ? -1 : (int)((kSlots >> (4 * lab)) & 15u);
     const bool writer = (lane & 1) == 0 && gslot >= 0;
-    const bool up16 = (lane & 16) != 0;
+    const float gscale = gslot >= 2 && gslot <= 4 ? 0.5f : 1.f;  // Sigma' sums are formed from 2 q
+    const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
     uint32_t tile;
     int sb;
     for (int it = 0; next_item(a.queue, a.counter, (uint32_t)a.V.n_tiles, NW, it, warp, lane, tile, sb); ++it) {
@@ -446,9 +448,12 @@ __global__ void __launch_bounds__(TW *TH) k_render_bwd(const BwdArgs a) {
         // the per-pixel factors of the channel pairs (red, n.x), (green, n.y), (blue, n.z) (FULL) or
         // (red, green) in kept / sent order for the level at offset 16: a lane with bit 16 clear keeps
         // the first of a pair and sends the second, the others the reverse
-        const float kc0 = FULL ? (up16 ? gN0 : gC0) : (up16 ? gC1 : gC0);
-        const float sc0 = FULL ? (up16 ? gC0 : gN0) : (up16 ? gC0 : gC1);
-        const float kc1 = up16 ? gN1 : gC1, sc1 = up16 ? gC1 : gN1;
+        // FULL: red and green, partners at offset 8, are exchanged as well in the lanes with bit 8 set
+        const float cr = FULL && up8 ? gC1 : gC0, cg = FULL && up8 ? gC0 : gC1;
+        const float nr = up8 ? gN1 : gN0, ng = up8 ? gN0 : gN1;
+        const float kc0 = FULL ? (up16 ? nr : cr) : (up16 ? gC1 : gC0);
+        const float sc0 = FULL ? (up16 ? cr : nr) : (up16 ? gC0 : gC1);
+        const float kc1 = up16 ? ng : cg, sc1 = up16 ? cg : ng;
         const float kc2 = up16 ? gN2 : gC2, sc2 = up16 ? gC2 : gN2;
         const uint32_t wend = __reduce_max_sync(0xffffffffu, lp);  // this warp replays [rg.x, wend)
         // transmittance before splat i and the channels accumulated up to and including
@@ -473,9 +478,11 @@ __global__ void __launch_bounds__(TW *TH) k_render_bwd(const BwdArgs a) {
                 const float4 r0 = slot[bit][0], r1 = slot[bit][1];
                 const float dx = fpx - r0.x, dy = fpy - r0.y;
                 PairEval pe;
-                const bool contrib =
-                    eval_pair_all(dx, dy, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, a.alpha_max, a.alpha_min, pe) &&
-                    c0 + (uint32_t)bit < lp;
+                // every lane evaluates the pair; its products 2b dy and c dy are kept for m below
+                const float b2dy = __fmul_rn(r0.w, dy), cdy = __fmul_rn(r1.x, dy);
+                const float Q = pair_q(dx, dy, r0.z, b2dy, cdy);
+                pair_alpha(Q, r1.z, r1.w, a.alpha_max, pe);
+                const bool contrib = Q <= r1.y && pe.alpha >= a.alpha_min && c0 + (uint32_t)bit < lp;
                 // Warp-uniform skip when no lane blends this splat; otherwise the body runs branch-free on
                 // every lane: a lane that does not blend takes alpha = 0, which leaves T and the running
                 // sums exactly as they were, and its values are selected to zero.
@@ -500,42 +507,43 @@ __global__ void __launch_bounds__(TW *TH) k_render_bwd(const BwdArgs a) {
                         behind = behind + gD * (Df - Da) + gN0 * (Nf0 - Na0) + gN1 * (Nf1 - Na1) +
                                  gN2 * (Nf2 - Na2);
                     }
-                    const float dal = contrib ? T * gc - (behind - gAT) * rcp_approx(1.f - al) : 0.f;
+                    const float dal = T * gc - (behind - gAT) * rcp_approx(1.f - al);  // used where contrib only
                     T = __fmul_rn(T, __fsub_rn(1.f, al));
                     const float o = r1.w, hb = r1.z;
                     const bool unclamped = contrib && pe.alpha_raw < a.alpha_max;
                     const float gop = unclamped ? dal * pe.G : 0.f;
-                    const float gG = unclamped ? dal * o : 0.f;
                     // G = exp(-p/2), p = Q^(beta/2): dG/dQ = -(beta/4) (p/Q) G, dG/dbeta = -(1/4) p ln(Q) G
-                    const bool qpos = contrib && pe.Q > 0.f;
-                    const float gp = gG * pe.p * pe.G;
-                    const float nq = qpos ? 0.5f * hb * gp * rcp_approx(pe.Q) : 0.f;  // -dL/dQ
+                    const bool qpos = unclamped && Q > 0.f;
+                    const float gp = dal * o * pe.p * pe.G;
+                    const float nq = qpos ? hb * gp * rcp_approx(Q) : 0.f;  // -2 dL/dQ
                     const float gbeta = qpos ? -0.25f * ln2 * gp * pe.lq : 0.f;
                     // Q = d^T C d with C = Sigma'^-1 and d = pixel - mean; with m = C d:
                     // dQ/dmean = -2 m and dQ/dSigma' = -m m^T (accumulated directly:
                     // going through the conic gradient would cancel for thin splats)
-                    const float mx = fmaf(r0.z, dx, 0.5f * r0.w * dy), my = fmaf(0.5f * r0.w, dx, r1.x * dy);
-                    // pairs (2 qx, 2 qy) and (qx mx, qy my), q = -dL/dQ m, from m in kept / sent order;
-                    // qx my = qy mx is S.xy either way. The channel pairs take their per-pixel factors
-                    // in that order already; the rest are swapped here.
+                    const float mx = __fmaf_rn(r0.z, dx, 0.5f * b2dy), my = __fmaf_rn(0.5f * r0.w, dx, cdy);
+                    // pairs (2 qx, 2 qy) and 2 (qx mx, qy my), q = -dL/dQ m, from m in kept / sent order;
+                    // qx my = qy mx is S.xy either way (the sums of Sigma' are halved at the end, exactly). The
+                    // channel pairs take their per-pixel factors in that order already; the rest are swapped here.
                     const float mk = up16 ? my : mx, ms = up16 ? mx : my;
                     const float qk = nq * mk, qs = nq * ms;
-                    keep[0] = 2.f * qk; send[0] = 2.f * qs;
-                    keep[1] = qk * mk; send[1] = qs * ms;
+                    constexpr int M = FULL ? 1 : 0;  // position of the mean
+                    keep[M] = qk; send[M] = qs;
+                    keep[M + 1] = qk * mk; send[M + 1] = qs * ms;
                     const float sxy = qk * ms;
-                    keep[2] = up16 ? gop : sxy; send[2] = up16 ? sxy : gop;
-                    keep[3] = kc0 * w; send[3] = sc0 * w;
+                    keep[M + 2] = up16 ? gop : sxy; send[M + 2] = up16 ? sxy : gop;
                     if (FULL) {
+                        keep[0] = kc0 * w; send[0] = sc0 * w;
                         keep[FULL ? 4 : 0] = kc1 * w; send[FULL ? 4 : 0] = sc1 * w;
                         keep[FULL ? 5 : 0] = kc2 * w; send[FULL ? 5 : 0] = sc2 * w;
                         const float gdep = gD * w;
                         keep[FULL ? 6 : 0] = up16 ? gdep : gbeta; send[FULL ? 6 : 0] = up16 ? gbeta : gdep;
                     } else {
+                        keep[3] = kc0 * w; send[3] = sc0 * w;
                         const float cb = gC2 * w;
                         keep[4] = up16 ? gbeta : cb; send[4] = up16 ? cb : gbeta;
                     }
                 }
-                const float sum = warp_reduce_split<NV>(keep, send, lane);
+                const float sum = gscale * warp_reduce_split<NV, FULL>(keep, send, lane);
                 if (writer) atomicAdd(a.g2d + 16 * (size_t)went[bit] + gslot, sum);
             }
             __syncwarp();
