@@ -29,6 +29,8 @@ constexpr int kK = GES_KNN_K;
 constexpr int kLsThreads = 32;
 constexpr int kLsChunk = 16;  // march samples whose densities a thread holds at once
 constexpr float kHalfLog2e = 0.72134752044448170f;
+constexpr float kLsGoneLog2 = 7.9657843f;  // log2 250
+constexpr float kLsFar = 1e5f;
 
 struct LsArgs {
     int n, m, n_views, n_steps;
@@ -118,9 +120,11 @@ __device__ __forceinline__ float term_at(const RayTerm &r, float t) {
     return r.o * ex2_approx(-kHalfLog2e * ex2_approx(r.hb * lg2_approx(Q)));
 }
 
-// One thread per pixel. The samples are taken kLsChunk at a time: each neighbour is put in
-// ray form once per chunk and its terms added to the chunk's densities in registers, then
-// the chunk is scanned for the first upward crossing (so nothing is staged in shared memory).
+// One thread per pixel. Bound by the special functions and the arithmetic of 16 x n_steps falloffs, so the
+// neighbours that add exactly 0 along the whole march are found first and left out (1.45M rays: 0.885 ->
+// 0.802 ms). The samples are taken kLsChunk at a time: each neighbour left is put in ray form once per chunk
+// and its terms added to the chunk's densities in registers, then the chunk is scanned for the first
+// upward crossing (so nothing is staged in shared memory).
 __global__ void __launch_bounds__(kLsThreads) k_ls_march(LsArgs a) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= a.m) return;
@@ -162,16 +166,33 @@ __global__ void __launch_bounds__(kLsThreads) k_ls_march(LsArgs a) {
     const float sigma = sqrtf(sig2);
     const int ns = a.n_steps;
     const float dt = 6.f * sigma / (float)(ns - 1);
+    // The neighbours whose terms are not all exactly 0 along the march (flat splats beside the ray mostly are: the
+    // falloff's exponent is past the end of float32). Q is least at the ray's closest approach in the splat's
+    // scaled axes; a neighbour is left out if its exponent there, P, is 250 or more where 175 already gives 0:
+    // that leaves Q 12 % (beta 6) to 105 % (beta 1), far more than its rounding moves it unless x0 lies more
+    // than kLsFar scales away, when the neighbour stays.
+    uint32_t live = 0;
+    for (int s = 0; s < kK; ++s) {
+        const int i = nbr(s);
+        if (i < 0) continue;
+        const RayTerm r = ray_term(load_rec(a.rec, i), p0, dir);
+        const float vv = fmaf(r.lv[0], r.lv[0], fmaf(r.lv[1], r.lv[1], r.lv[2] * r.lv[2]));
+        const float lv = fmaf(r.l0[0], r.lv[0], fmaf(r.l0[1], r.lv[1], r.l0[2] * r.lv[2]));
+        const float t = fminf(fmaxf(-lv / vv, -3.f * sigma), 3.f * sigma);
+        const float l0 = fmaf(t, r.lv[0], r.l0[0]), l1 = fmaf(t, r.lv[1], r.l0[1]), l2 = fmaf(t, r.lv[2], r.l0[2]);
+        const float Q = fmaf(l0, l0, fmaf(l1, l1, l2 * l2));
+        const float far = fmaxf(fabsf(r.l0[0]), fmaxf(fabsf(r.l0[1]), fabsf(r.l0[2])));
+        const bool gone = r.hb * lg2_approx(Q) >= kLsGoneLog2 && far <= kLsFar && r.o < 3e38f;
+        if (!gone) live |= 1u << s;  // (also where a comparison met a NaN)
+    }
     float tprev = 0.f, dprev = 0.f, tstar = 0.f;
     bool found = false;
     for (int j0 = 0; j0 < ns && !found; j0 += kLsChunk) {
         float d[kLsChunk];
 #pragma unroll
         for (int j = 0; j < kLsChunk; ++j) d[j] = 0.f;
-        for (int s = 0; s < kK; ++s) {
-            const int i = nbr(s);
-            if (i < 0) continue;
-            const RayTerm r = ray_term(load_rec(a.rec, i), p0, dir);
+        for (uint32_t m = live; m; m &= m - 1u) {
+            const RayTerm r = ray_term(load_rec(a.rec, nbr(__ffs(m) - 1)), p0, dir);
 #pragma unroll
             for (int j = 0; j < kLsChunk; ++j) d[j] += term_at(r, fmaf((float)(j0 + j), dt, -3.f * sigma));
         }
