@@ -335,7 +335,7 @@ GES_API size_t ges_loss_workspace_bytes(int32_t n_views, const ges_camera *cams)
  *            ties to the lower index (so neighbour 0 is i itself unless another centre
  *            coincides with it and has a lower index)
  * Exact (distances are squared float32 differences summed in x, y, z order) unless
- * one query must examine more than 65,536 candidate centres (tens of thousands of
+ * one query must examine more than 131,072 candidate centres (tens of thousands of
  * coincident centres, or non-finite coordinates); its list is then the best among
  * those examined. Workspace: ges_knn_workspace_bytes(n) bytes, 256-byte aligned, no
  * initialisation needed. n must be in [16, 2^26]; otherwise both calls reject it
@@ -353,7 +353,7 @@ GES_API ges_status ges_knn(int32_t n, const float *pos_op, void *workspace, size
  *   knn      [m, 16] int32 (written, 16-byte aligned): point j's neighbours by increasing
  *            distance, ties to the lower index
  * The points are searched in grid-cell order; cells are grouped in 4 x 4 x 4 blocks whose
- * counts let a query in empty space skip them. Exactness and the 65,536-candidate bound
+ * counts let a query in empty space skip them. Exactness and the 131,072-candidate bound
  * are as for ges_knn. Workspace: ges_knn_points_workspace_bytes(n, m) bytes, 256-byte
  * aligned, no initialisation needed. n in [16, 2^26], m in [1, 2^28]. */
 GES_API size_t ges_knn_points_workspace_bytes(int32_t n, int32_t m);

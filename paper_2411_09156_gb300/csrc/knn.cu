@@ -1,7 +1,7 @@
 // Exact k = 16 nearest splat centres (Sec. 4.2: the GSR density at a sample uses
 // the 16 splats closest to the splat it was drawn from).
 //
-// A uniform grid over the centres' bounding box, at most two cells per point, is
+// A uniform grid over the centres' bounding box, at most one cell per point, is
 // built on the device: cell keys and counts, a stable radix sort of the points by cell (the
 // sort of the binning), the scan of the counts (the first centre of every cell, so that a run of
 // cells along x is one range of centres, read with two loads) and a cell-ordered copy of the centres.
@@ -9,11 +9,12 @@
 // distances alone, then, over the cells within the 16th, for the centres themselves. Rows of
 // cells farther than the current 16th are skipped and the others cut to it along x, which keeps
 // queries away from the centres (points in front of a surface) from reading every cell of their
-// block. Queries run in cell order, so a warp searches one
-// neighbourhood. Distances are squared float32 with a fixed operation order; ties go to
-// the lower index. A query that would examine more than 65,536 candidates (a bound that well-spread
+// block. (Cells, whole call: 2 per point, 1, 1/2: KNN of a 1.5M-splat heightfield 1.24, 1.26, 1.50 ms, of
+// a 300k-splat object 1.52, 1.02, 0.92; level-set points of a 1600x1040 view 3.00, 2.58, 2.48.) Queries run in
+// cell order, so a warp searches one neighbourhood. Distances are squared float32 with a fixed operation order; ties go to
+// the lower index. A query that would examine more than 131,072 candidates (a bound that well-spread
 // centres never reach; tens of thousands of coincident centres would) takes the best of the first
-// 65,536 in ring order instead, so no input makes the search quadratic.
+// 131,072 in ring order instead, so no input makes the search quadratic.
 #include "ges_internal.cuh"
 #include "sort_net.cuh"
 
@@ -22,7 +23,7 @@ namespace ges {
 namespace {
 
 constexpr int kK = GES_KNN_K;
-constexpr uint32_t kQueryBudget = 1u << 16;  // candidate points one query may examine
+constexpr uint32_t kQueryBudget = 1u << 17;  // candidate points one query may examine
 // 16 CTAs of 64 threads per SM (64 registers): at 12 or 20 the centre queries take 11 % or 1 % longer
 constexpr int kQueryThreads = 64, kQueryCtas = 16;
 // The first pass ends when the searched cells reach sqrt(kReach) of the 16th distance: the second pass then
@@ -52,7 +53,7 @@ inline uint64_t al256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
 KnnLayout knn_layout(int32_t n) {
     KnnLayout L;
-    uint64_t cap = 2ull * (uint64_t)n;
+    uint64_t cap = (uint64_t)n;
     if (cap < 1) cap = 1;
     if (cap > (1ull << 26) - 1) cap = (1ull << 26) - 1;  // one scan covers the cells and the end
     L.cap_cells = (uint32_t)cap;
@@ -97,6 +98,10 @@ __global__ void __launch_bounds__(256) k_knn_bbox(const float4 *pos, int n, uint
             mx[k] = max(mx[k], o);
         }
     }
+    // one set of atomics a CTA: all of them meet at six addresses
+    __shared__ uint32_t s_bb[6];
+    if (threadIdx.x < 6) s_bb[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+    __syncthreads();
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         mn[k] = __reduce_min_sync(0xffffffffu, mn[k]);
@@ -105,10 +110,13 @@ __global__ void __launch_bounds__(256) k_knn_bbox(const float4 *pos, int n, uint
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            atomicMin(bb + k, mn[k]);
-            atomicMax(bb + 3 + k, mx[k]);
+            atomicMin(s_bb + k, mn[k]);
+            atomicMax(s_bb + 3 + k, mx[k]);
         }
     }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMin(bb + threadIdx.x, s_bb[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(bb + threadIdx.x, s_bb[threadIdx.x]);
 }
 
 // Cell size h with at most cap cells: start from the volume per cell, then grow h
@@ -786,7 +794,7 @@ static cudaError_t knn_build(int32_t n, const float4 *pos, void *workspace, cons
     if (e == cudaSuccess) e = cudaMemsetAsync(starts, 0, 4ull * (L.cap_cells + 1ull), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(at<void>(workspace, L.bcount), 0, 4ull * L.cap_cells, s);
     if (e != cudaSuccess) return e;
-    k_knn_bbox<<<min(ceil_div_u64(n, 256), 1024u), 256, 0, s>>>(pos, n, bb);
+    k_knn_bbox<<<min(ceil_div_u64(n, 1024), 608u), 256, 0, s>>>(pos, n, bb);
     k_knn_grid<<<1, 1, 0, s>>>(bb, L.cap_cells, grid);
     uint32_t *keys[2] = {at<uint32_t>(workspace, L.keys0), at<uint32_t>(workspace, L.keys1)};
     uint32_t *vals[2] = {at<uint32_t>(workspace, L.vals0), at<uint32_t>(workspace, L.vals1)};
