@@ -92,26 +92,32 @@ __device__ __forceinline__ void warp_tile_tests(const TileJob &J, int lane, int 
 
 // ST: the colour storage (Params::color_storage), a template parameter so that each storage
 // gets its own register allocation.
+// A warp takes 32 splats in one view, or 16 in two (`pairs`). With a splat's views side by side in the warp (16
+// views: 2 splats a warp) every record array was written in runs of two records, far apart, and every read of a
+// camera parameter, which lies in constant memory at the lane's view, took one access per view: 16 views of
+// 3M splats 4.71 ms, 8 views of 1.5M 0.84, 8 of 100k 0.24; now 2.82, 0.71, 0.09.
 template <int ST>
-__global__ void __launch_bounds__(32, 32) k_preprocess(PreArgs a) {
+__global__ void __launch_bounds__(32, 32) k_preprocess(PreArgs a, bool pairs) {
     const uint32_t NV = (uint32_t)a.V.n_views;
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;  // n * NV < 2^31 (host check)
     const int lane = threadIdx.x & 31;
-    const bool live = t < (uint32_t)a.count * NV;
+    // block k of the NV that share 32 splats: view k of all of them, or half of them in two views
+    const uint32_t run = blockIdx.x / NV, k = blockIdx.x - run * NV;
+    const bool two = pairs && (k | 1u) < NV;
+    const uint32_t v = two ? (k & ~1u) + (uint32_t)(lane & 1) : k;
+    const uint32_t il = 32u * run + (two ? 16u * (k & 1u) + (uint32_t)(lane >> 1) : (uint32_t)lane);
+    const bool live = il < (uint32_t)a.count;
     const int tw = a.V.tile_w, th = a.V.tile_h;
     const int lw = __ffs(tw) - 1, lh = __ffs(th) - 1;  // tile sides are powers of two
-    uint32_t i = 0, v = 0;
+    uint32_t i = 0;
     size_t e = 0;
     float z32 = 0.f, ext_x = 0.f, ext_y = 0.f;
     bool visible = false;
     TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
     uint32_t rect = 0, rdim = 0;
     if (live) {
-        const uint32_t il = t / NV;
-        v = t - il * NV;
         i = (uint32_t)a.first + il;
         e = (size_t)v * a.n + i;
-        if (v == 0 && a.P.sh_degree >= 0) {
+        if (!(two && (lane & 1)) && a.P.sh_degree >= 0) {
             // the splat's colour coefficients (first and last byte: at most two lines for SH3) into
             // L2 while the projection runs, one lane per splat
             const int bytes = a.P.n_coeffs * 3 * (ST == 0 ? 4 : 2);
@@ -597,13 +603,16 @@ __global__ void __launch_bounds__(32, 28) k_preprocess_bwd(PreBwdArgs a) {
 
 cudaError_t launch_preprocess(const PreArgs &a, cudaStream_t s) {
     if (a.count <= 0) return cudaSuccess;
-    const long long threads = (long long)a.count * a.V.n_views;
     // one warp per CTA: the warps share nothing but the SM, so a warp whose tile tests end early
     // frees its slot at once (0.93 -> 0.83 ms against CTAs of 8 warps)
-    const unsigned grid = (unsigned)((threads + 31) / 32);
-    if (a.P.color_storage == 1) k_preprocess<1><<<grid, 32, 0, s>>>(a);
-    else if (a.P.color_storage == 2) k_preprocess<2><<<grid, 32, 0, s>>>(a);
-    else k_preprocess<0><<<grid, 32, 0, s>>>(a);
+    const unsigned grid = ceil_div_u64((uint64_t)a.count, 32) * (unsigned)a.V.n_views;
+    // Two views a warp where the splat's coefficients are the larger part of its reads (they are fetched once per
+    // warp). 8 views of 1.5M splats, pairs against single views: 192 B (SH3) 784, 895 us; 108 B (SH2) 806,
+    // 843; 96 B (SH3 in 16 bits) 751, 751; RGB 682, 671; 100k splats: 106, 104; 106, 100; 104, 94; 102, 90.
+    const bool pairs = a.P.sh_degree >= 0 && a.P.n_coeffs * 3 * (a.P.color_storage == 0 ? 4 : 2) > 96;
+    if (a.P.color_storage == 1) k_preprocess<1><<<grid, 32, 0, s>>>(a, pairs);
+    else if (a.P.color_storage == 2) k_preprocess<2><<<grid, 32, 0, s>>>(a, pairs);
+    else k_preprocess<0><<<grid, 32, 0, s>>>(a, pairs);
     return cudaGetLastError();
 }
 
