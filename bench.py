@@ -329,13 +329,16 @@ def other_workloads(cfg, args, flush, rank: int, world: int) -> dict:
     return out
 
 
+def knn_build_launches(n: int) -> int:
+    """Kernels of the grid build over n centres: bounding box, grid, cell keys and counts, the 3 of
+    their scan, the gather and 5 per 8-bit radix pass."""
+    return 7 + 5 * ((max(1, (n - 1).bit_length()) + 7) // 8)
+
+
 def levelset_launches(n: int) -> int:
-    """Kernels one ges_levelset call launches: start points, splat records, the grid build
-    (bounding box, grid, cell keys, ranges, 5 per 8-bit radix pass), the query keys and their
-    radix sort, the point queries and the march."""
-    p_n = ((2 * n - 1).bit_length() + 7) // 8
-    p_q = ((2 * n).bit_length() + 7) // 8
-    return 8 + 5 * p_n + 5 * p_q
+    """Kernels one ges_levelset call launches: start points, splat records, the grid build, the
+    query keys and their radix sort, the point queries and the march."""
+    return 5 + knn_build_launches(n) + 5 * ((n.bit_length() + 7) // 8)
 
 
 def profile_traffic(kernel: str):
@@ -687,7 +690,7 @@ def main():
                "gsr_fwd_bwd_ms": fb_ms, "gsr_fwd_ms": fwd_ms, "knn_ms": knn_ms,
                "losses": [round(float(x), 6) for x in losses.cpu().tolist()],
                "sampling": "one sample per splat, z ~ N(0, I), neighbours = the splat's 16 nearest centres",
-               "gpu_launches": args.steps * ((6 + 5 * (((2 * n - 1).bit_length() + 7) // 8)) + 3 + 4)}
+               "gpu_launches": args.steps * (knn_build_launches(n) + 1 + 3 + 4)}
         del kws, knn, gws, gg
         torch.cuda.empty_cache()
 

@@ -161,12 +161,13 @@ GES_API ges_status ges_preprocess_range(int32_t n, int32_t first, int32_t count,
  * the last ges_preprocess on `proj` produced (sum of tiles touched). */
 GES_API ges_status ges_instance_count(const void *proj, size_t proj_bytes, uint64_t *count, void *stream);
 
-/* S5: binning. Sorts entries by float32 depth (stable LSD radix sort), emits one
- * (global tile, entry) instance per listed tile in depth order, sorts the
- * instances by tile (stable, so depth order is kept within a tile) and finds
- * each tile's [start, end) range. With cfg->persistent it also builds the
- * longest-first tile queue. If the instances exceed the capacity `bins` was
- * sized for, the lists are truncated and GES_ERR_CAPACITY is recorded. */
+/* S5: binning. Counts the instances (entry, listed tile) of every tile, scans the
+ * counts into one segment per tile ([start, end) in concatenated tile order), writes
+ * every instance to its tile's segment and sorts each segment by (float32 depth,
+ * entry). With cfg->persistent it also builds the longest-first tile queue. If the
+ * instances exceed the capacity `bins` was sized for, the lists are truncated (each
+ * is then some of its tile's instances, in depth order) and GES_ERR_CAPACITY is
+ * recorded. */
 GES_API ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges_config *cfg, void *proj,
                    size_t proj_bytes, void *bins, size_t bins_bytes, void *stream);
 

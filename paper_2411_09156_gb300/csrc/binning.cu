@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t *in, uint32_
     if (threadIdx.x == 0) partials[blockIdx.x] = tot;
 }
 
-// One CTA of 1024 threads scans up to kScanMaxPartials tile sums; writes the grand total.
-__global__ void __launch_bounds__(1024) k_scan_partials(uint32_t *partials, uint32_t np, uint32_t *total) {
+// One CTA of 1024 threads scans up to kScanMaxPartials tile sums.
+__global__ void __launch_bounds__(1024) k_scan_partials(uint32_t *partials, uint32_t np) {
     __shared__ uint32_t s_warp[33];
     constexpr int PER = kScanMaxPartials / 1024;
     uint32_t v[PER];
@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(1024) k_scan_partials(uint32_t *partials, uint
         if (idx < np) partials[idx] = run;
         run += v[k];
     }
-    if (threadIdx.x == 0 && total) *total = tot;
 }
 
 __global__ void __launch_bounds__(256) k_scan_down(const uint32_t *in, uint32_t *out, uint32_t n,
@@ -124,31 +123,23 @@ __global__ void __launch_bounds__(256) k_scan_down(const uint32_t *in, uint32_t 
     }
 }
 
-cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *partials, uint32_t *total,
-                           cudaStream_t s) {
+cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *partials, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     const uint32_t nb = ceil_div_u64(n, kScanTile);
     if (nb > (uint32_t)kScanMaxPartials) return cudaErrorInvalidValue;
     k_scan_reduce<<<nb, 256, 0, s>>>(in, n, partials);
-    k_scan_partials<<<1, 1024, 0, s>>>(partials, nb, total);
+    k_scan_partials<<<1, 1024, 0, s>>>(partials, nb);
     k_scan_down<<<nb, 256, 0, s>>>(in, out, n, partials);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ radix sort
-// Count source: n_dev (device, clamped to cap) if given, else n_host.
-__device__ __forceinline__ uint32_t live_count(const uint32_t *n_dev, uint32_t n_host) {
-    return n_dev ? *n_dev : n_host;
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *keys, const uint32_t *n_dev,
-                                                            uint32_t n_host, int shift, uint32_t nblocks,
-                                                            uint32_t *hist) {
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *keys, uint32_t n, int shift,
+                                                            uint32_t nblocks, uint32_t *hist) {
     __shared__ uint32_t s_h[kSortThreads / 32][256];
     const int warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < (kSortThreads / 32) * 256; k += kSortThreads) (&s_h[0][0])[k] = 0u;
     __syncthreads();
-    const uint32_t n = live_count(n_dev, n_host);
     const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
     if (base < n) {
         uint32_t kk[kSortItems];
@@ -178,8 +169,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *key
 // the scanned digit-major histogram.
 __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(const uint32_t *keys_in, const uint32_t *vals_in,
                                                                uint32_t *keys_out, uint32_t *vals_out,
-                                                               const uint32_t *n_dev, uint32_t n_host, int shift,
-                                                               uint32_t nblocks, const uint32_t *hist_scanned) {
+                                                               uint32_t n, int shift, uint32_t nblocks,
+                                                               const uint32_t *hist_scanned) {
     constexpr int NW = kSortThreads / 32;
     __shared__ uint32_t s_cnt[NW][256];
     __shared__ uint32_t s_dstart[256], s_gstart[256];
@@ -188,7 +179,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(const uint32_
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < NW * 256; k += kSortThreads) (&s_cnt[0][0])[k] = 0u;
     __syncthreads();
-    const uint32_t n = live_count(n_dev, n_host);
     const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
     if (base >= n) return;  // uniform for the CTA
     const uint32_t nvalid = (uint32_t)min((uint64_t)kSortTile, (uint64_t)n - base);
@@ -258,27 +248,25 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(const uint32_
         const uint32_t k = s_keys[i];
         const uint32_t d = (k >> shift) & 0xffu;
         const uint32_t pos = s_gstart[d] + (i - s_dstart[d]);
-        if (keys_out) keys_out[pos] = k;
+        keys_out[pos] = k;
         vals_out[pos] = s_vals[i];
     }
 }
 
-// Sorts (keys, vals) on bits [0, bits) with ceil(bits/8) passes, ping-ponging
-// between buffer 0 and 1; the result lands in buffer (passes % 2). vals[0] may be
-// NULL for "value = index". Keys are always written (tile ranges need them).
-cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], bool iota_vals, const uint32_t *n_dev,
-                       uint32_t n_host_max, int bits, uint32_t *hist, uint32_t *partials, cudaStream_t s) {
-    const uint32_t nblocks = ceil_div_u64(n_host_max > 0 ? n_host_max : 1, kSortTile);
+// Sorts (keys[0][i], i) on key bits [0, bits) with ceil(bits/8) passes, ping-ponging
+// between buffer 0 and 1; the result lands in buffer (passes % 2).
+cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], uint32_t n, int bits, uint32_t *hist,
+                       uint32_t *partials, cudaStream_t s) {
+    const uint32_t nblocks = ceil_div_u64(n > 0 ? n : 1, kSortTile);
     const int passes = (bits + 7) / 8;
     for (int p = 0; p < passes; ++p) {
         const int in = p & 1, out = in ^ 1;
         const int shift = 8 * p;
-        k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(keys[in], n_dev, n_host_max, shift, nblocks, hist);
-        cudaError_t e = exclusive_scan(hist, hist, 256u * nblocks, partials, nullptr, s);
+        k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(keys[in], n, shift, nblocks, hist);
+        cudaError_t e = exclusive_scan(hist, hist, 256u * nblocks, partials, s);
         if (e != cudaSuccess) return e;
-        k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(keys[in], (p == 0 && iota_vals) ? nullptr : vals[in],
-                                                        keys[out], vals[out], n_dev, n_host_max, shift, nblocks,
-                                                        hist);
+        k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(keys[in], p == 0 ? nullptr : vals[in], keys[out], vals[out], n,
+                                                        shift, nblocks, hist);
     }
     return cudaGetLastError();
 }

@@ -109,12 +109,6 @@ constexpr int kScanMaxPartials = 1024 * 16;
 
 inline uint32_t ceil_div_u64(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
-inline int bits_for(uint32_t v) {  // bits needed to hold values 0..v-1
-    int b = 0;
-    while (b < 32 && (1ull << b) < (uint64_t)v) ++b;
-    return b;
-}
-
 // Tile lists are sorted by CTAs: up to kCtaList entries by one CTA of 512 threads (or a part of one), up to
 // kBigList by one CTA of 1024, longer ones in chunks of at most kBigList.
 constexpr uint32_t kCtaList = 4096, kBigList = 16384;
@@ -256,11 +250,6 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
     f32x2 r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
 
@@ -538,12 +527,11 @@ struct BwdArgs {
 cudaError_t launch_preprocess(const PreArgs &a, cudaStream_t s);
 cudaError_t launch_preprocess_bwd(const PreBwdArgs &a, cudaStream_t s);
 cudaError_t launch_bin(const BinArgs &a, cudaStream_t s);
-// Stable LSD radix sort of (key, value) pairs on bits [0, bits), 8 bits a pass (binning.cu).
-cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], bool iota_vals, const uint32_t *n_dev,
-                       uint32_t n_host_max, int bits, uint32_t *hist, uint32_t *partials, cudaStream_t s);
+// Stable LSD radix sort of (keys[0][i], i) on key bits [0, bits), 8 bits a pass (binning.cu).
+cudaError_t radix_sort(uint32_t *keys[2], uint32_t *vals[2], uint32_t n, int bits, uint32_t *hist,
+                       uint32_t *partials, cudaStream_t s);
 // Exclusive scan of n uint32 (binning.cu); partials: ceil(n / kScanTile) + 1 words. In place is allowed.
-cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *partials, uint32_t *total,
-                           cudaStream_t s);
+cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, uint32_t n, uint32_t *partials, cudaStream_t s);
 cudaError_t launch_render_fwd(const FwdArgs &a, cudaStream_t s);
 cudaError_t launch_render_bwd(const BwdArgs &a, cudaStream_t s);
 bool tile_shape_supported(int tw, int th);

@@ -800,9 +800,9 @@ static cudaError_t knn_build(int32_t n, const float4 *pos, void *workspace, cons
     uint32_t *vals[2] = {at<uint32_t>(workspace, L.vals0), at<uint32_t>(workspace, L.vals1)};
     k_knn_keys<<<ceil_div_u64(n, 256), 256, 0, s>>>(pos, n, grid, keys[0], starts, at<uint32_t>(workspace, L.bcount));
     // cell counts -> first centre of each cell, and the end
-    e = exclusive_scan(starts, starts, L.cap_cells + 1u, at<uint32_t>(workspace, L.partials), nullptr, s);
+    e = exclusive_scan(starts, starts, L.cap_cells + 1u, at<uint32_t>(workspace, L.partials), s);
     if (e != cudaSuccess) return e;
-    e = radix_sort(keys, vals, true, nullptr, (uint32_t)n, L.bits, at<uint32_t>(workspace, L.hist),
+    e = radix_sort(keys, vals, (uint32_t)n, L.bits, at<uint32_t>(workspace, L.hist),
                    at<uint32_t>(workspace, L.partials), s);
     if (e != cudaSuccess) return e;
     const int res = ((L.bits + 7) / 8) & 1;
@@ -829,7 +829,7 @@ cudaError_t knn_points_run(int32_t n, const float4 *pos, int32_t m, const float4
     uint32_t *vals[2] = {at<uint32_t>(qws, Q.vals0), at<uint32_t>(qws, Q.vals1)};
     k_knn_point_keys<<<ceil_div_u64(m, 256), 256, 0, s>>>(pts, m, at<KnnGrid>(workspace, L.grid),
                                                           (uint32_t)((1ull << Q.bits) - 1), keys[0]);
-    e = radix_sort(keys, vals, true, nullptr, (uint32_t)m, Q.bits, at<uint32_t>(qws, Q.hist),
+    e = radix_sort(keys, vals, (uint32_t)m, Q.bits, at<uint32_t>(qws, Q.hist),
                    at<uint32_t>(qws, Q.partials), s);
     if (e != cudaSuccess) return e;
     const int res = ((Q.bits + 7) / 8) & 1;
