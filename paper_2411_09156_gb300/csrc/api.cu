@@ -266,6 +266,7 @@ ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges
     a.pairs = at<unsigned long long>(bins, L.pairs);
     a.ranges = at<uint2>(bins, L.ranges);
     a.queue = at<uint32_t>(bins, L.queue);
+    a.buckets = at<uint32_t>(bins, L.buckets);
     a.aux = at<TileAux>(bins, L.aux);
     a.counts = at<uint32_t>(bins, L.counts);
     a.lists = at<uint4>(bins, L.lists);

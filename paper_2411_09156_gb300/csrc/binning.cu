@@ -449,7 +449,7 @@ __device__ __forceinline__ int length_bucket(uint32_t len) {
     return b < 0 ? 0 : b;
 }
 
-// Tile index, first part: each CTA's instances and, for the queue, the tiles per length bucket. A CTA takes
+// Tile index, first part: each CTA's instances and, for the queue, its tiles per length bucket. A CTA takes
 // `per` consecutive tiles (a multiple of 1024).
 __global__ void __launch_bounds__(1024) k_tile_sums(const BinArgs a, uint32_t per) {
     __shared__ uint32_t s_warp[33], s_bucket[kLptBuckets];
@@ -468,8 +468,8 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const BinArgs a, uint32_t pe
     uint32_t tot;
     block_excl_scan(sum, s_warp, tot);
     if (threadIdx.x == 0) a.aux->partial[blockIdx.x] = tot;
-    if (a.build_queue && threadIdx.x < kLptBuckets && s_bucket[threadIdx.x])
-        atomicAdd(&a.aux->bucket[threadIdx.x], s_bucket[threadIdx.x]);
+    if (a.build_queue && threadIdx.x < kLptBuckets)
+        a.buckets[(size_t)blockIdx.x * kLptBuckets + threadIdx.x] = s_bucket[threadIdx.x];
 }
 
 // Sort class of a segment of n instances at `start`, clipped to the capacity: -1 nothing to sort, kListClasses too
@@ -480,25 +480,43 @@ __device__ __forceinline__ int seg_class(const BinArgs &a, uint32_t start, uint3
 }
 
 // Tile index, second part: each tile's range clipped to the capacity, its segments' starts (in place of their
-// counts) and their places in the sort classes' lists or chunk jobs, and the tile's place in the queue.
+// counts) and their places in the sort classes' lists or chunk jobs, and the tile's place in the queue. Within a
+// bucket the queue keeps the tiles' order: the render backward takes the tiles in the queue's order and adds their
+// gradients with float atomics, and the sums of a thin splat's Sigma' cancel so far that another order moves its
+// gradients by 3e-5. With places taken by atomics across the CTAs the order varied from run to run.
 __global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t per) {
-    __shared__ uint32_t s_warp[33], s_prefix[kLptBuckets], s_cnt[kLptBuckets], s_base[kLptBuckets];
+    __shared__ uint32_t s_warp[33], s_all[kLptBuckets], s_next[kLptBuckets];
+    __shared__ uint32_t s_rank[32][kLptBuckets];  // tiles of a bucket per warp, then its first place
     __shared__ uint32_t s_cls[kListClasses], s_cls_base[kListClasses];
     const uint32_t n_tiles = (uint32_t)a.V.n_tiles, t0 = blockIdx.x * per, tid = threadIdx.x, S = a.slabs;
+    const int lane = (int)(tid & 31u), warp = (int)(tid >> 5);
     if (blockIdx.x == 0 && tid == 0) {
         const unsigned long long t = *a.total;
         a.header[0] = t >= 0xffffffffull ? 0u : (uint32_t)(t < a.cap ? t : a.cap);
     }
     uint32_t run, tot;
     block_excl_scan(tid < blockIdx.x ? a.aux->partial[tid] : 0u, s_warp, run);  // at most kTileBlocks CTAs before
-    if (a.build_queue) {
-        const uint32_t p = block_excl_scan(tid < kLptBuckets ? a.aux->bucket[tid] : 0u, s_warp, tot);
-        if (tid < kLptBuckets) s_prefix[tid] = p;
+    if (a.build_queue) {  // the buckets' first places for this CTA: all longer buckets, then the CTAs before
+        if (tid < kLptBuckets) s_all[tid] = s_next[tid] = 0u;
+        __syncthreads();
+        const uint32_t b = tid % kLptBuckets;
+        uint32_t all = 0, before = 0;
+        for (uint32_t c = tid / kLptBuckets; c < gridDim.x; c += 1024u / kLptBuckets) {
+            const uint32_t n = a.buckets[(size_t)c * kLptBuckets + b];
+            all += n;
+            if (c < blockIdx.x) before += n;
+        }
+        atomicAdd(&s_all[b], all);
+        atomicAdd(&s_next[b], before);
+        __syncthreads();
+        const uint32_t p = block_excl_scan(tid < kLptBuckets ? s_all[tid] : 0u, s_warp, tot);
+        if (tid < kLptBuckets) s_next[tid] += p;
     }
     for (uint32_t k0 = 0; k0 < per; k0 += 1024) {
         const uint32_t t = t0 + k0 + tid;
         if (t0 + k0 >= n_tiles) break;  // uniform for the CTA
-        if (tid < kLptBuckets) s_cnt[tid] = 0u;
+        if (a.build_queue)
+            for (uint32_t k = tid; k < 32u * kLptBuckets; k += 1024u) s_rank[k / kLptBuckets][k % kLptBuckets] = 0u;
         if (tid < kListClasses) s_cls[tid] = 0u;
         __syncthreads();
         uint32_t c = 0;
@@ -506,15 +524,16 @@ __global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t p
             for (uint32_t q = 0; q < S; ++q) c += a.counts[(size_t)t * S + q];
         const uint32_t start = run + block_excl_scan(c, s_warp, tot);
         run += tot;
-        uint32_t slot = 0;
-        int bucket = 0;
+        const int bucket = t < n_tiles ? length_bucket(c) : kLptBuckets;
+        uint32_t rank = 0;
+        if (a.build_queue) {
+            const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
+            rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
+            if (rank == 0u && t < n_tiles) s_rank[warp][bucket] = (uint32_t)__popc(peers);
+        }
         if (t < n_tiles) {
             const uint64_t s = min((uint64_t)start, a.cap), e = min((uint64_t)start + c, a.cap);
             a.ranges[t] = e > s ? make_uint2((uint32_t)s, (uint32_t)e) : make_uint2(0u, 0u);
-            if (a.build_queue) {
-                bucket = length_bucket(c);
-                slot = atomicAdd(&s_cnt[bucket], 1u);
-            }
             // the tile's segments: their starts replace their counts
             uint32_t at = start;
             for (uint32_t q = 0; q < S; ++q) {
@@ -530,7 +549,16 @@ __global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t p
             s_cls_base[tid] = s_cls[tid] ? atomicAdd(&a.aux->n_list[tid], s_cls[tid]) : 0u;
             s_cls[tid] = 0u;
         }
-        if (a.build_queue && tid < kLptBuckets) s_base[tid] = s_cnt[tid] ? atomicAdd(&a.aux->bucket_cur[tid], s_cnt[tid]) : 0u;
+        if (a.build_queue && tid < kLptBuckets) {
+            uint32_t next = s_next[tid];
+#pragma unroll
+            for (int w = 0; w < 32; ++w) {
+                const uint32_t n = s_rank[w][tid];
+                s_rank[w][tid] = next;
+                next += n;
+            }
+            s_next[tid] = next;
+        }
         __syncthreads();
         if (t < n_tiles) {
             uint32_t at = start;
@@ -550,7 +578,7 @@ __global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t p
                 at = end;
             }
         }
-        if (a.build_queue && t < n_tiles) a.queue[s_prefix[bucket] + s_base[bucket] + slot] = t;
+        if (a.build_queue && t < n_tiles) a.queue[s_rank[warp][bucket] + rank] = t;
         __syncthreads();
     }
 }
@@ -939,8 +967,7 @@ cudaError_t launch_bin(const BinArgs &a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     // 2. segments, ranges, sort classes, queue
-    const uint32_t per = 1024u * ceil_div_u64(n_tiles, 1024ull * kTileBlocks);
-    const uint32_t nblk = ceil_div_u64(n_tiles, per);
+    const uint32_t per = tiles_per_cta(n_tiles), nblk = tile_ctas(n_tiles);
     k_tile_sums<<<nblk, 1024, 0, s>>>(a, per);
     k_tile_index<<<nblk, 1024, 0, s>>>(a, per);
     if (a.n == 0) return cudaGetLastError();

@@ -116,23 +116,26 @@ constexpr int kLptBuckets = 128;   // list-length buckets of the longest-first q
 constexpr int kListClasses = 4;    // <= 256, <= 1024, <= kCtaList, <= kBigList entries
 constexpr uint32_t kTileBlocks = 512;  // most CTAs of the tile-index kernels
 
+// Tiles per CTA of the tile-index kernels (a multiple of 1024), and their CTAs.
+inline uint32_t tiles_per_cta(uint32_t n_tiles) { return 1024u * ceil_div_u64(n_tiles, 1024ull * kTileBlocks); }
+inline uint32_t tile_ctas(uint32_t n_tiles) { return ceil_div_u64(n_tiles, tiles_per_cta(n_tiles)); }
+
 // Counters of the tile index, cleared by every ges_bin together with the tile counts after them.
 struct TileAux {
     uint32_t partial[kTileBlocks];     // instances of each CTA's tiles
-    uint32_t bucket[kLptBuckets];      // tiles per list-length bucket
-    uint32_t bucket_cur[kLptBuckets];  // queue slots taken per bucket
     uint32_t n_list[kListClasses];     // segments per sort class
     uint32_t n_jobs;                   // chunks of longer ones
     uint32_t depth_hi[kMaxViews], depth_lo_inv[kMaxViews];  // greatest depth bits of a view's entries, and of ~bits
 };
 
 // bins: [header 256][instance tile cap x 4][instance entry cap x 4][unsorted instances cap x 8][ranges T x 8]
-//       [queue T][TileAux, counts of the G = T x slabs segments x 4][class lists 4 x G x 16][chunk jobs x 16]
+//       [queue T][tiles per length bucket of each tile-index CTA]
+//       [TileAux, counts of the G = T x slabs segments x 4][class lists 4 x G x 16][chunk jobs x 16]
 //       [places: CTAs per view x G x 4]
 // header: u32 n_inst (instances actually listed) at 0, u32 queue counters at 4 and 8, u64 count of
 // the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval).
 struct BinsLayout {
-    uint64_t tile, entry, pairs, ranges, queue, aux, counts, lists, jobs, places, bytes;
+    uint64_t tile, entry, pairs, ranges, queue, buckets, aux, counts, lists, jobs, places, bytes;
     uint32_t n_tiles;
 };
 
@@ -197,6 +200,7 @@ inline BinsLayout bins_layout(int32_t n, const ViewSet &V, uint64_t cap) {
     L.pairs = off; off = align256(off + cap * 8);
     L.ranges = off; off = align256(off + (uint64_t)n_tiles * 8);
     L.queue = off; off = align256(off + (uint64_t)n_tiles * 4);
+    L.buckets = off; off = align256(off + 4ull * kLptBuckets * tile_ctas(n_tiles));
     L.aux = off; L.counts = off + sizeof(TileAux); off = align256(L.counts + n_segs * 4);
     L.lists = off; off = align256(off + n_segs * 16 * kListClasses);
     // a list of more than kBigList entries has ceil(len / kBigList) < 2 len / kBigList chunks
@@ -477,6 +481,7 @@ struct BinArgs {
     unsigned long long *pairs;  // depth bits << 32 | entry, grouped by tile
     uint2 *ranges;
     uint32_t *queue;
+    uint32_t *buckets;  // [CTAs of the tile-index kernels][kLptBuckets]: tiles per length bucket
     TileAux *aux;
     uint32_t *counts;  // instances per segment (tile x slabs + slab), then the next free slot of it
     uint4 *lists;      // [kListClasses][segments]: start, end, tile, -
