@@ -927,9 +927,12 @@ static int sm_count() {
 
 template <bool EMIT, bool SHARED, bool SLABS>
 static cudaError_t launch_instances_t(const BinArgs &a, uint32_t grid, uint32_t threads, int smem, cudaStream_t s) {
-    if (smem) {  // on every call: the attribute belongs to the current device
+    if (SHARED) {
+        // on every call: the attribute belongs to the current device. Always the same bound: with this call's own size
+        // a thread binning a smaller view could lower it between another's attribute and launch
         const cudaError_t e = cudaFuncSetAttribute(k_instances<EMIT, SHARED, SLABS>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(uint32_t) * kSharedCounters));
         if (e != cudaSuccess) return e;
     }
     k_instances<EMIT, SHARED, SLABS><<<grid, threads, smem, s>>>(a);
