@@ -165,9 +165,9 @@ GES_API ges_status ges_instance_count(const void *proj, size_t proj_bytes, uint6
  * counts into one segment per tile ([start, end) in concatenated tile order), writes
  * every instance to its tile's segment and sorts each segment by (float32 depth,
  * entry). With cfg->persistent it also builds the longest-first tile queue. If the
- * instances exceed the capacity `bins` was sized for, the lists are truncated (each
- * is then some of its tile's instances, in depth order) and GES_ERR_CAPACITY is
- * recorded. */
+ * instances exceed the capacity `bins` was sized for, the nearest are kept, the first
+ * `capacity` of all views' instances in the order of (depth, entry, tile), and
+ * GES_ERR_CAPACITY is recorded. */
 GES_API ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges_config *cfg, void *proj,
                    size_t proj_bytes, void *bins, size_t bins_bytes, void *stream);
 

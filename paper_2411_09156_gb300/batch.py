@@ -193,11 +193,11 @@ class BatchPlan:
 
     def launches_per_step(self) -> int:
         """Kernels of this library launched by one step (cudaMemsetAsync nodes not counted)."""
-        # binning: tile counts and appends (with splats; a depth-range pass before them where the entries are
-        # 512 or more a tile), two index launches, then the list sorts a list of this length may need
+        # binning: counters, tile counts and appends (with splats; a depth-range pass before them where the entries
+        # are 512 or more a tile), two index launches, then the list sorts a list of this length may need
         dense = self.n * len(self.cams) >= 512 * int(self.rast.layout().n_tiles)
         longest = min(self.n, self.capacity)
-        binning = 2 if self.n == 0 else 4 + dense + 1 + (longest > 4096) + (longest > 16384)
+        binning = 3 if self.n == 0 else 5 + dense + 1 + (longest > 4096) + (longest > 16384)
         return 1 + binning + 1 + 1 + 1 + (2 if self.target is not None else 0)
 
 

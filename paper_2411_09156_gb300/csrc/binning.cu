@@ -11,6 +11,8 @@
 // 128 -> 55; 1.5M at 1600x1040 313 -> 280; 4 views of 300k 216 -> 160; 8 views of 1.5M (34.7M
 // instances) 1488 -> 1150. What bounds it there: the scattered 8-byte appends (425 us) and the sorts' shared-memory
 // traffic (430 us). Only lists far beyond a CTA got slower (1.5M splats in one 16x16 view: 224 -> 308 us).
+#include <cooperative_groups.h>
+
 #include "ges_internal.cuh"
 #include "sort_net.cuh"
 #include "tile_tests.cuh"
@@ -284,6 +286,103 @@ __device__ __forceinline__ uint32_t select_bit(uint32_t m, uint32_t k) {
     return pos;
 }
 
+// The tile tests of entry e of view v (box in binrec's first half b0).
+__device__ __forceinline__ TileJob tile_job(const BinArgs &a, int v, size_t e, const uint4 b0, int lw, int lh) {
+    TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
+    const float4 r0 = a.rec[4 * e], r1 = a.rec[4 * e + 1];
+    int x0, x1, y0, y1;
+    pixel_box(r0.x, r0.y, __uint_as_float(b0.x), __uint_as_float(b0.y), a.V.width[v], a.V.height[v], x0, x1, y0, y1);
+    if (x0 <= x1 && y0 <= y1)
+        J = TileJob{r0.x, r0.y, r0.z, r0.w, r1.x, __frcp_rn(r0.z), __frcp_rn(r1.x), __fmul_rn(r1.y, kSupportMargin),
+                    (uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16),
+                    (uint32_t)((x1 >> lw) - (x0 >> lw) + 1) * (uint32_t)((y1 >> lh) - (y0 >> lh) + 1)};
+    return J;
+}
+
+// First kernel of a ges_bin: clears the counters and, if there are more instances than the capacity, finds where the
+// lists end: the instances kept are the first `cap` of all in the order of (depth, entry, tile), so what is lost is the
+// farthest of every view. A radix selection over the entries' 64-bit keys (depth, entry), weighted by their tiles, by
+// the CTAs of one cluster, whose barrier and shared memory it needs; it leaves in the header the key of the entry
+// that the capacity cuts, the first tile that this entry loses, and a 1 (header zero: nothing is cut).
+// Without an overflow it costs about what the memory clear that it replaced did (2.6 us; the whole binning of a
+// 1.5M-splat view 280 -> 286 us with it and the ordered queue); with one, six passes over the records by one cluster
+// (8 views of 1.5M splats: 6 ms of binning instead of 1.2; one 100k-splat view: 139 us instead of 80).
+constexpr int kCutCtas = 8;
+__global__ void __cluster_dims__(kCutCtas, 1, 1) __launch_bounds__(1024) k_bin_begin(const BinArgs a, uint4 *clear,
+                                                                                     uint64_t n_clear) {
+    const uint32_t t = threadIdx.x, lane = t & 31u, rank = blockIdx.x;
+    for (uint64_t i = rank * 1024u + t; i < n_clear; i += kCutCtas * 1024u) clear[i] = make_uint4(0u, 0u, 0u, 0u);
+    const unsigned long long total = *a.total;
+    if (total <= a.cap || total >= 0xffffffffull) return;  // the same for the cluster
+    constexpr int kDigit = 11, kBins = 1 << kDigit;
+    __shared__ uint32_t s_bins[kBins], s_warp[33], s_digit, s_before;
+    __shared__ uint4 s_jobs[kJobWords * 32];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint64_t n_entries = (uint64_t)a.n * (uint64_t)a.n_views;
+    unsigned long long prefix = 0;
+    uint32_t left = (uint32_t)a.cap;  // instances kept among the keys that begin with `prefix`
+    for (int shift = 64; shift > 0;) {
+        const int bits = shift < kDigit ? shift : kDigit, above = shift;
+        shift -= bits;
+        for (uint32_t k = t; k < kBins; k += 1024u) s_bins[k] = 0u;
+        if (t == 0) s_digit = kBins;
+        __syncthreads();
+#pragma unroll 4
+        for (uint64_t e = rank * 1024u + t; e < n_entries; e += kCutCtas * 1024u) {
+            const uint4 b0 = __ldg(a.binrec + 2 * e);
+            const unsigned long long key = ((unsigned long long)b0.w << 32) | e;
+            if (b0.z && (above == 64 || key >> above == prefix))
+                atomicAdd(&s_bins[(uint32_t)(key >> shift) & ((1u << bits) - 1u)], b0.z);
+        }
+        cluster.sync();
+        uint32_t c0 = 0, c1 = 0, tot;
+        for (uint32_t r = 0; r < kCutCtas; ++r) {
+            const uint32_t *b = cluster.map_shared_rank(s_bins, r);
+            c0 += b[2 * t];
+            c1 += b[2 * t + 1];
+        }
+        const uint32_t first = block_excl_scan(c0 + c1, s_warp, tot);
+        if (left >= first && left - first < c0 + c1) {  // one thread
+            const bool second = left - first >= c0;
+            s_digit = 2u * t + (second ? 1u : 0u);
+            s_before = first + (second ? c0 : 0u);
+        }
+        cluster.sync();  // every CTA is past the bins, and this CTA's threads see the digit
+        const uint32_t digit = s_digit, before = s_before;
+        if (digit == kBins) return;  // (the entries hold fewer instances than the total says; the same for the cluster)
+        prefix = (prefix << bits) | digit;
+        left -= before;
+        __syncthreads();  // the digit is reset after every thread has it
+    }
+    if (rank != 0 || t >= 32u) return;
+    // the key's entry keeps its first `left` tiles: find its hit number `left`
+    const uint32_t e = (uint32_t)prefix;
+    const int v = (int)(e / (uint32_t)a.n), tiles_x = a.V.tiles_x[v];
+    const uint4 b0 = __ldg(a.binrec + 2 * (size_t)e), b1 = __ldg(a.binrec + 2 * (size_t)e + 1);
+    const uint32_t tbase = (uint32_t)a.V.tile_base[v], bw = b1.z & 0xffffu, bh = b1.z >> 16;
+    auto cut_at = [&](uint32_t tx, uint32_t ty) {  // called by one lane
+        *reinterpret_cast<unsigned long long *>(a.header + kCutWord) = prefix;
+        a.header[kCutWord + 2] = tbase + ty * (uint32_t)tiles_x + tx;
+        a.header[kCutWord + 3] = 1u;
+        set_error(a.err, kErrCapacity);
+    };
+    if (bw * bh <= 32u) {
+        const uint32_t bit = select_bit(b1.x, left);
+        if (lane == 0) cut_at((b1.y & 0xffffu) + bit % bw, (b1.y >> 16) + bit / bw);
+        return;
+    }
+    const int tw = a.V.tile_w, th = a.V.tile_h, lw = __ffs(tw) - 1, lh = __ffs(th) - 1;
+    TileJob J = tile_job(a, v, e, b0, lw, lh);
+    if (lane != 0) J.nbox = 0u;
+    uint32_t seen = 0;
+    warp_tile_rounds(J, (int)lane, lw, lh, tw, th, s_jobs, 0u, 1u,
+                     [&](uint32_t hits, uint32_t, uint32_t, uint32_t, int tx, int ty, uint32_t, bool hit) {
+                         if (hit && seen + (uint32_t)__popc(hits & ((1u << lane) - 1u)) == left) cut_at((uint32_t)tx, (uint32_t)ty);
+                         seen += (uint32_t)__popc(hits);
+                     });
+}
+
 // The instances of a warp's 32 entries, each listed tile of each entry once: on_instance(global tile, depth bits,
 // entry) is called by one lane each. Entries whose box has at most 32 tiles are expanded from their hit masks
 // by the whole warp, 32 instances a round (instance j goes to the entry whose prefix interval holds j, binary
@@ -329,15 +428,7 @@ __device__ __forceinline__ void warp_instances(const BinArgs &a, int v, uint32_t
     const int tw = a.V.tile_w, th = a.V.tile_h;
     const int lw = __ffs(tw) - 1, lh = __ffs(th) - 1;  // tile sides are powers of two
     TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
-    if (big) {
-        const float4 r0 = a.rec[4 * e], r1 = a.rec[4 * e + 1];
-        int x0, x1, y0, y1;
-        pixel_box(r0.x, r0.y, __uint_as_float(b0.x), __uint_as_float(b0.y), a.V.width[v], a.V.height[v], x0, x1, y0, y1);
-        if (x0 <= x1 && y0 <= y1)
-            J = TileJob{r0.x, r0.y, r0.z, r0.w, r1.x, __frcp_rn(r0.z), __frcp_rn(r1.x), __fmul_rn(r1.y, kSupportMargin),
-                        (uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16),
-                        (uint32_t)((x1 >> lw) - (x0 >> lw) + 1) * (uint32_t)((y1 >> lh) - (y0 >> lh) + 1)};
-    }
+    if (big) J = tile_job(a, v, e, b0, lw, lh);
     warp_tile_rounds(J, lane, lw, lh, tw, th, jobs, part, a.parts,
                      [&](uint32_t, uint32_t, uint32_t, uint32_t, int tx, int ty, uint32_t owner, bool hit) {
                          const uint32_t depth = __shfl_sync(0xffffffffu, b0.w, owner);
@@ -354,7 +445,8 @@ __device__ __forceinline__ void warp_instances(const BinArgs &a, int v, uint32_t
 // the append of the same entries starts there, so a CTA's instances of a tile land side by side.
 // SLABS: the tiles' segments are split by depth.
 template <bool EMIT, bool SHARED, bool SLABS>
-__global__ void __launch_bounds__(kInstThreads) k_instances(const BinArgs a) {
+__global__ void __launch_bounds__(kInstThreads, EMIT || SLABS ? 3 : 4) k_instances(const BinArgs a) {
+    const bool cut = a.header[kCutWord + 3] != 0u;  // (read beside the total)
     if (*a.total >= 0xffffffffull) {  // uint32 positions would wrap: no lists
         if (!EMIT && blockIdx.x == 0 && threadIdx.x == 0) set_error(a.err, kErrCapacity);
         return;
@@ -379,7 +471,7 @@ __global__ void __launch_bounds__(kInstThreads) k_instances(const BinArgs a) {
         if (!SLABS) return tile;
         return tile * S + min((uint32_t)max((int)((__uint_as_float(depth) - z0) * per_z), 0), S - 1u);
     };
-    auto each = [&](auto &&on_instance) {
+    auto each_of = [&](auto &&on_instance) {
         for (uint32_t w0 = i0 + (uint32_t)warp * 32u; w0 < i1; w0 += blockDim.x) {
             const uint32_t i = w0 + (uint32_t)lane;
             const size_t e = (size_t)v * a.n + i;
@@ -393,9 +485,21 @@ __global__ void __launch_bounds__(kInstThreads) k_instances(const BinArgs a) {
             warp_instances(a, v, tiles, b0, b1, e, s_jobs[warp], lane, part, on_instance);
         }
     };
+    // those that the capacity's cut keeps, in a loop of its own: the ordinary one needs no depths to count
+    auto each = [&](auto &&on_instance) {
+        if (!cut) {
+            each_of(on_instance);
+            return;
+        }
+        each_of([&](uint32_t tile, uint32_t depth, uint32_t e) {
+            const unsigned long long key = ((unsigned long long)depth << 32) | e,
+                                     last = *reinterpret_cast<const unsigned long long *>(a.header + kCutWord);
+            if (key < last || (key == last && tile < a.header[kCutWord + 2])) on_instance(tile, depth, e);
+        });
+    };
     auto append = [&](uint32_t slot, uint32_t depth, uint32_t e) {
         if (slot < a.cap) a.pairs[slot] = ((unsigned long long)depth << 32) | e;
-        else set_error(a.err, kErrCapacity);
+        else set_error(a.err, kErrCapacity);  // (counts beyond the total only: the cut keeps within the capacity)
     };
     if (SHARED) {
         uint32_t *place = a.places + (size_t)row * ((size_t)a.V.n_tiles * S) + tbase;
@@ -951,7 +1055,11 @@ static cudaError_t launch_instances(const BinArgs &a, bool shared, uint32_t grid
 
 cudaError_t launch_bin(const BinArgs &a, cudaStream_t s) {
     const uint32_t n_tiles = (uint32_t)a.V.n_tiles;
-    cudaError_t e = cudaMemsetAsync(a.aux, 0, sizeof(TileAux) + sizeof(uint32_t) * (size_t)n_tiles * a.slabs, s);
+    // 0. counters (aux is 256-byte aligned inside bins and its array ends on such a boundary), the capacity's cut
+    static_assert(sizeof(TileAux) % 16 == 0, "cleared with the counts after it, 16 bytes at a time");
+    k_bin_begin<<<kCutCtas, 1024, 0, s>>>(a, reinterpret_cast<uint4 *>(a.aux),
+                                          (sizeof(TileAux) + sizeof(uint32_t) * (uint64_t)n_tiles * a.slabs + 15u) / 16u);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int sms = sm_count();
     // 1. instances per tile: counted in shared memory while a view's counters fit; a CTA takes as many entries as

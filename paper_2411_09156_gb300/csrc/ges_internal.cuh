@@ -126,6 +126,7 @@ struct TileAux {
     uint32_t n_list[kListClasses];     // segments per sort class
     uint32_t n_jobs;                   // chunks of longer ones
     uint32_t depth_hi[kMaxViews], depth_lo_inv[kMaxViews];  // greatest depth bits of a view's entries, and of ~bits
+    uint32_t pad[3];
 };
 
 // bins: [header 256][instance tile cap x 4][instance entry cap x 4][unsorted instances cap x 8][ranges T x 8]
@@ -133,7 +134,9 @@ struct TileAux {
 //       [TileAux, counts of the G = T x slabs segments x 4][class lists 4 x G x 16][chunk jobs x 16]
 //       [places: CTAs per view x G x 4]
 // header: u32 n_inst (instances actually listed) at 0, u32 queue counters at 4 and 8, u64 count of
-// the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval).
+// the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval), the capacity's cut
+// (u64 key, u32 tile, u32 1) at 32 (zero: nothing cut).
+constexpr int kCutWord = 8;
 struct BinsLayout {
     uint64_t tile, entry, pairs, ranges, queue, buckets, aux, counts, lists, jobs, places, bytes;
     uint32_t n_tiles;
