@@ -508,7 +508,10 @@ __device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid
                     if (xa < 0 || xb >= G.dims[0]) continue;
                     const uint2 rg = row_within(q, G, starts, y, z, xa, xb, left);
                     examined += rg.y - rg.x;
-                    if (examined > kQueryBudget) break;
+                    if (examined > kQueryBudget) {
+                        bd[kK - 1] = -1.f;  // given up: no further row is read
+                        break;
+                    }
                     for_centres(rg, spos, [&](float4 o) { insert_dist(dist2(q.p, o), bd); });
                 }
             }
@@ -546,7 +549,7 @@ __device__ __forceinline__ void ball_centres(const CellPoint &q, const KnnGrid &
             if (left < 0.f) continue;
             const uint2 rg = row_within(q, G, starts, y, z, 0, G.dims[0] - 1, left);
             examined += rg.y - rg.x;
-            if (examined > kQueryBudget) break;
+            if (examined > kQueryBudget) return;
             for_centres(rg, spos, [&](float4 o) {
                 const float d = dist2(q.p, o);
                 if (d <= bound) add_found(f, d, __float_as_uint(o.w));
@@ -557,6 +560,22 @@ __device__ __forceinline__ void ball_centres(const CellPoint &q, const KnnGrid &
 __device__ __forceinline__ CellPoint cell_point(float4 p, const KnnGrid &G) {
     return CellPoint{p, cell_axis(p.x, G.lo[0], G.inv_h, G.dims[0]), cell_axis(p.y, G.lo[1], G.inv_h, G.dims[1]),
                      cell_axis(p.z, G.lo[2], G.inv_h, G.dims[2])};
+}
+
+// Whether a point has all coordinates: else no distance to it is a number, and its list stays empty.
+__device__ __forceinline__ bool has_coordinates(float4 p) { return p.x == p.x && p.y == p.y && p.z == p.z; }
+
+// Whether all distances from p overflow: they bound nothing, and the bounded searches, which then end with the first 16
+// centres they meet, serve.
+__device__ __forceinline__ bool all_infinite(float4 p, const KnnGrid &G) {
+    const float pc[3] = {p.x, p.y, p.z};
+    float d2 = 0.f;  // squared distance to the grid's box
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float g = fmaxf(fmaxf(G.lo[k] - G.slack - pc[k], pc[k] - (G.lo[k] + (float)G.dims[k] * G.h + G.slack)), 0.f);
+        d2 = fmaf(g, g, d2);
+    }
+    return !(d2 < __int_as_float(0x7f800000));
 }
 
 __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_query(const float4 *spos, const uint32_t *starts,
@@ -572,11 +591,15 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_query(const f
 #pragma unroll
     for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
     uint32_t examined = 0;
-    near_distances(q, G, starts, spos, 1 << 20, kReach, examined, bd);
     Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
-    if (examined <= kQueryBudget) {
-        examined = 0;
-        ball_centres(q, G, starts, spos, bd[kK - 1], examined, f);
+    if (all_infinite(p, G)) {
+        examined = kQueryBudget + 1u;
+    } else if (has_coordinates(p)) {
+        near_distances(q, G, starts, spos, 1 << 20, kReach, examined, bd);
+        if (examined <= kQueryBudget) {
+            examined = 0;
+            ball_centres(q, G, starts, spos, bd[kK - 1], examined, f);
+        }
     }
     if (examined > kQueryBudget) {
         ring_search_bounded(p, gp, starts, spos, out);
@@ -697,8 +720,12 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
     const float4 p = pts[r];
     int4 *out = reinterpret_cast<int4 *>(knn + (size_t)r * kK);
     Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
-    if (p.w != 0.f) {
+    if (p.w != 0.f && has_coordinates(p)) {
         const KnnGrid G = *gp;
+        if (all_infinite(p, G)) {
+            block_search_bounded(p, gp, starts, spos, reinterpret_cast<int32_t *>(out));
+            return;
+        }
         float bd[kK];
 #pragma unroll
         for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
@@ -715,7 +742,10 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
                 q, G, starts, bcount, max(max(G.dims[0], G.dims[1]), G.dims[2]), [&]() { return bd[kK - 1]; },
                 [&](uint2 rg) {
                     examined += rg.y - rg.x;
-                    if (examined > kQueryBudget) return;
+                    if (examined > kQueryBudget) {  // given up: the walk ends (it would read every row of the
+                        bd[kK - 1] = -1.f;          // grid where the distances never narrow the bound)
+                        return;
+                    }
                     for_centres(rg, spos, [&](float4 o) { insert_dist(dist2(p, o), bd); });
                 });
         }
