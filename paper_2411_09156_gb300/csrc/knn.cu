@@ -479,7 +479,8 @@ __device__ __forceinline__ float row_gap(const CellPoint &q, const KnnGrid &G, i
 // The centres of the cells [x0, x1] of row (y, z) that lie within sqrt(left) of q.p along x.
 __device__ __forceinline__ uint2 row_within(const CellPoint &q, const KnnGrid &G, const uint32_t *starts, int y, int z,
                                             int x0, int x1, float left) {
-    const float w = sqrt_above(left) + G.slack;
+    // (the whole row where `left` is no number: an infinite bound less an infinite distance)
+    const float w = fminf(sqrt_above(left), 3e38f) + G.slack;
     x0 = max(x0, min(cell_axis(q.p.x - w, G.lo[0], G.inv_h, G.dims[0]), q.cx));
     x1 = min(x1, max(cell_axis(q.p.x + w, G.lo[0], G.inv_h, G.dims[0]), q.cx));
     const int row = G.dims[0] * (y + G.dims[1] * z);
