@@ -489,16 +489,23 @@ __device__ __forceinline__ uint2 row_within(const CellPoint &q, const KnnGrid &G
 
 // First pass: the 27 cells around q's, then further rings (at most `rings` in all) until bd holds 16
 // distances and the searched cells reach sqrt(reach) of the 16th in every open direction. The middle rows come
-// first, so that the bound soon leaves most of the others out. Returns whether bd holds 16 distances.
+// first, so that the bound soon leaves most of the others out. Returns whether bd holds 16 distances. MANY: as many rings
+// as it takes.
+template <bool MANY>
 __device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid &G, const uint32_t *starts,
                                                const float4 *spos, int rings, float reach, uint32_t &examined,
                                                float (&bd)[kK]) {
+    // Many rings: their rows reach no further along an axis than the grid's farther end, and once the x faces of the
+    // searched cells are outside the grid only a ring's outer rows are new. The rings of a query far from any others (a
+    // line's outlier takes 2,048) would else run over thousands of rows each that are not there or searched already.
+    const int most_y = MANY ? max(q.cy, G.dims[1] - 1 - q.cy) : 1 << 20, most_z = MANY ? max(q.cz, G.dims[2] - 1 - q.cz) : 1 << 20;
     for (int R = 1; R <= rings && examined <= kQueryBudget; ++R) {
         const int x0 = max(q.cx - R, 0), x1 = min(q.cx + R, G.dims[0] - 1);
-        for (int zi = 0; zi <= 2 * R; ++zi) {
+        const bool outer = MANY && R > 1 && q.cx - R < 0 && q.cx + R >= G.dims[0];
+        for (int zi = outer && R > most_y ? 2 * R - 1 : 0; zi <= 2 * min(R, most_z); ++zi) {
             const int z = q.cz + ((zi & 1) ? -((zi + 1) >> 1) : (zi >> 1));
             if (z < 0 || z >= G.dims[2]) continue;
-            for (int yi = 0; yi <= 2 * R; ++yi) {
+            for (int yi = outer && abs(z - q.cz) < R ? 2 * R - 1 : 0; yi <= 2 * min(R, most_y); ++yi) {
                 const int y = q.cy + ((yi & 1) ? -((yi + 1) >> 1) : (yi >> 1));
                 if (y < 0 || y >= G.dims[1]) continue;
                 const float left = bd[kK - 1] - row_gap(q, G, y, z);
@@ -531,7 +538,7 @@ __device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid
         face(q.cz + R < G.dims[2] - 1, (G.lo[2] + (float)(q.cz + R + 1) * G.h) - q.p.z);
         b = fmaxf(b, 0.f);
         if (all || (full && reach * bd[kK - 1] <= b * b)) return full;
-        if (R > 1 && R < rings && rings <= kNearRings && examined == 0u) return false;  // empty space: blocks skip it
+        if (!MANY && R > 1 && R < rings && examined == 0u) return false;  // empty space: blocks skip it
     }
     return bd[kK - 1] < __int_as_float(0x7f800000);
 }
@@ -596,7 +603,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_query(const f
     if (all_infinite(p, G)) {
         examined = kQueryBudget + 1u;
     } else if (has_coordinates(p)) {
-        near_distances(q, G, starts, spos, 1 << 20, kReach, examined, bd);
+        near_distances<true>(q, G, starts, spos, 1 << 20, kReach, examined, bd);
         if (examined <= kQueryBudget) {
             examined = 0;
             ball_centres(q, G, starts, spos, bd[kK - 1], examined, f);
@@ -733,7 +740,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
         uint32_t examined = 0;
         const CellPoint q = cell_point(p, G);
         // most queries lie within a few cells of 16 centres; the others walk blocks, which skip empty space
-        const bool near = near_distances(q, G, starts, spos, kNearRings, kReach, examined, bd);
+        const bool near = near_distances<false>(q, G, starts, spos, kNearRings, kReach, examined, bd);
         int rings = 0;
         if (!near && examined <= kQueryBudget) {
 #pragma unroll
