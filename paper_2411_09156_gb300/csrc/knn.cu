@@ -24,6 +24,12 @@ namespace {
 
 constexpr int kK = GES_KNN_K;
 constexpr uint32_t kQueryBudget = 1u << 17;  // candidate points one query may examine
+// A query with more candidates than this in the 27 cells around it leaves the two passes for one pass of pair
+// insertion: its nearest tie (coincident centres), and each pass costs a distance per candidate. 50,000 coincident
+// centres: 26.8 ms with two passes that searched the whole column at each tie, 13.6 with the column's greatest pair kept,
+// 7.3 in one pass (before the two passes: 6.6); 100,000: 75.7, 27.9, 15.1 (9.0 with half the budget). Ordinary queries
+// examine a few hundred.
+constexpr uint32_t kTwoPassMost = 2048;
 // 16 CTAs of 64 threads per SM (64 registers): at 12 or 20 the centre queries take 11 % or 1 % longer
 constexpr int kQueryThreads = 64, kQueryCtas = 16;
 // The first pass ends when the searched cells reach sqrt(kReach) of the 16th distance: the second pass then
@@ -258,11 +264,18 @@ __device__ __forceinline__ void ring_search(float4 p, const KnnGrid &G, const ui
             const int cell = cx + G.dims[0] * (cy + G.dims[1] * cz);
             scan_cell(p, row_range(starts, cell, cell), spos, examined, bd, bi);
         };
-        // the cells at Chebyshev distance `ring` from the query's cell
-        for (int cz = z0; cz <= z1; ++cz) {
+        // the cells at Chebyshev distance `ring` from the query's cell; where neither x face lies in the grid, of the
+        // inner rows there is nothing to see, nor of the inner planes where no y face does (a line in one cell of a
+        // flat grid has 2,048 rings)
+        const bool no_x = ring > 0 && c[0] - ring < 0 && c[0] + ring >= G.dims[0];
+        const bool no_xy = no_x && c[1] - ring < 0 && c[1] + ring >= G.dims[1];
+        for (int cz = no_xy ? c[2] - ring : z0; cz <= z1; cz += no_xy ? 2 * ring : 1) {
+            if (cz < 0) continue;
             const float gz = gap(2, cz);
             if (gz * gz > bd[kK - 1]) continue;
-            for (int cy = y0; cy <= y1; ++cy) {
+            const bool faces = no_x && abs(cz - c[2]) < ring;
+            for (int cy = faces ? c[1] - ring : y0; cy <= y1; cy += faces ? 2 * ring : 1) {
+                if (cy < 0) continue;
                 const float gy = gap(1, cy);
                 const float gyz = fmaf(gy, gy, gz * gz);
                 if (gyz > bd[kK - 1]) continue;
@@ -399,11 +412,23 @@ __device__ __forceinline__ void insert_dist(float d, float (&bd)[kK]) {
     bd[0] = fminf(bd[0], d);
 }
 
-// A thread's table column: up to kK candidates (distance, index), unsorted, `stride` apart.
+// A thread's table column: up to kK candidates (distance, index), unsorted, `stride` apart; once a further one came, its
+// greatest pair and where that lies (-1 until then).
 struct Found {
     uint2 *col;
     int stride, n;
+    uint2 w;
+    int worst;
 };
+
+__device__ __forceinline__ void find_worst(Found &f) {
+    f.worst = 0;
+    f.w = f.col[0];
+    for (int k = 1; k < kK; ++k) {
+        const uint2 c = f.col[k * f.stride];
+        if (c.x > f.w.x || (c.x == f.w.x && c.y > f.w.y)) { f.w = c; f.worst = k; }
+    }
+}
 
 // Adds (d, id); a full column replaces its greatest pair if (d, id) comes before it.
 __device__ __forceinline__ void add_found(Found &f, float d, uint32_t id) {
@@ -413,13 +438,10 @@ __device__ __forceinline__ void add_found(Found &f, float d, uint32_t id) {
         ++f.n;
         return;
     }
-    int worst = 0;
-    uint2 w = f.col[0];
-    for (int k = 1; k < kK; ++k) {
-        const uint2 c = f.col[k * f.stride];
-        if (c.x > w.x || (c.x == w.x && c.y > w.y)) { w = c; worst = k; }
-    }
-    if (db < w.x || (db == w.x && id < w.y)) f.col[worst * f.stride] = make_uint2(db, id);
+    if (f.worst < 0) find_worst(f);
+    if (db > f.w.x || (db == f.w.x && id >= f.w.y)) return;  // ties of many centres end here
+    f.col[f.worst * f.stride] = make_uint2(db, id);
+    find_worst(f);
 }
 
 // The column sorted by (distance, index), as indices; missing entries -1.
@@ -516,7 +538,8 @@ __device__ __forceinline__ bool near_distances(const CellPoint &q, const KnnGrid
                     if (xa < 0 || xb >= G.dims[0]) continue;
                     const uint2 rg = row_within(q, G, starts, y, z, xa, xb, left);
                     examined += rg.y - rg.x;
-                    if (examined > kQueryBudget) {
+                    if (examined > (MANY && R == 1 ? kTwoPassMost : kQueryBudget)) {
+                        examined = kQueryBudget + 1u;
                         bd[kK - 1] = -1.f;  // given up: no further row is read
                         break;
                     }
@@ -599,7 +622,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_query(const f
 #pragma unroll
     for (int k = 0; k < kK; ++k) bd[k] = __int_as_float(0x7f800000);
     uint32_t examined = 0;
-    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
+    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0, make_uint2(0u, 0u), -1};
     if (all_infinite(p, G)) {
         examined = kQueryBudget + 1u;
     } else if (has_coordinates(p)) {
@@ -727,7 +750,7 @@ __global__ void __launch_bounds__(kQueryThreads, kQueryCtas) k_knn_points(const 
     const uint32_t r = __ldg(order + r0);
     const float4 p = pts[r];
     int4 *out = reinterpret_cast<int4 *>(knn + (size_t)r * kK);
-    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0};
+    Found f = {&s_found[0][threadIdx.x], kQueryThreads, 0, make_uint2(0u, 0u), -1};
     if (p.w != 0.f && has_coordinates(p)) {
         const KnnGrid G = *gp;
         if (all_infinite(p, G)) {
