@@ -30,7 +30,7 @@ constexpr int kLsThreads = 32;
 constexpr int kLsChunk = 16;  // march samples whose densities a thread holds at once
 constexpr float kHalfLog2e = 0.72134752044448170f;
 constexpr float kLsGoneLog2 = 7.9657843f;  // log2 250
-constexpr float kLsFar = 1e5f;
+constexpr float kLsFar = 1e5f, kLsMostHb = 10.f;
 
 struct LsArgs {
     int n, m, n_views, n_steps;
@@ -168,9 +168,10 @@ __global__ void __launch_bounds__(kLsThreads) k_ls_march(LsArgs a) {
     const float dt = 6.f * sigma / (float)(ns - 1);
     // The neighbours whose terms are not all exactly 0 along the march (flat splats beside the ray mostly are: the
     // falloff's exponent is past the end of float32). Q is least at the ray's closest approach in the splat's
-    // scaled axes; a neighbour is left out if its exponent there, P, is 250 or more where 175 already gives 0:
-    // that leaves Q 12 % (beta 6) to 105 % (beta 1), far more than its rounding moves it unless x0 lies more
-    // than kLsFar scales away, when the neighbour stays.
+    // scaled axes (beta > 0: P grows with Q); a neighbour is left out if its exponent there, P, is 250 or more where
+    // 175 already gives 0. That leaves Q 0.71 / beta of itself, 3.6 % at kLsMostHb's beta 20, the largest that is
+    // left out. Rounding moves the approach along the ray by a few float32 units of x0's distance, at most 0.1
+    // scales at kLsFar (beyond it the neighbour stays), and Q, least there, by the square of that: 0.6 %.
     uint32_t live = 0;
     for (int s = 0; s < kK; ++s) {
         const int i = nbr(s);
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kLsThreads) k_ls_march(LsArgs a) {
         const float l0 = fmaf(t, r.lv[0], r.l0[0]), l1 = fmaf(t, r.lv[1], r.l0[1]), l2 = fmaf(t, r.lv[2], r.l0[2]);
         const float Q = fmaf(l0, l0, fmaf(l1, l1, l2 * l2));
         const float far = fmaxf(fabsf(r.l0[0]), fmaxf(fabsf(r.l0[1]), fabsf(r.l0[2])));
-        const bool gone = r.hb * lg2_approx(Q) >= kLsGoneLog2 && far <= kLsFar && r.o < 3e38f;
+        const bool gone = r.hb * lg2_approx(Q) >= kLsGoneLog2 && r.hb > 0.f && r.hb <= kLsMostHb && far <= kLsFar && r.o < 3e38f;
         if (!gone) live |= 1u << s;  // (also where a comparison met a NaN)
     }
     float tprev = 0.f, dprev = 0.f, tstar = 0.f;
