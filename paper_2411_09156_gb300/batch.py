@@ -193,12 +193,21 @@ class BatchPlan:
 
     def launches_per_step(self) -> int:
         """Kernels of this library launched by one step (cudaMemsetAsync nodes not counted)."""
-        # binning: counters, tile counts and appends (with splats; a depth-range pass before them where the entries
-        # are 512 or more a tile), two index launches, then the list sorts a list of this length may need
-        dense = self.n * len(self.cams) >= 512 * int(self.rast.layout().n_tiles)
-        longest = min(self.n, self.capacity)
-        binning = 3 if self.n == 0 else 5 + dense + 1 + (longest > 4096) + (longest > 16384)
+        binning = binning_launches(self.n, self.rast.sizes, self.cfg.tile_w, self.cfg.tile_h, self.capacity)
         return 1 + binning + 1 + 1 + 1 + (2 if self.target is not None else 0)
+
+
+def binning_launches(n: int, sizes, tile_w: int, tile_h: int, capacity: int) -> int:
+    """Kernels one ges_bin launches for n splats in views of these sizes: the counters and two index launches;
+    with splats, the tile counts, the appends and the sort of ordinary lists too, a depth-range pass where
+    tiles are split by depth (512 entries or more a tile, and twice the largest view's tiles within the
+    24,576 counters of a CTA's shared memory), and the sorts that a list of up to min(n, capacity) may need."""
+    if n == 0:
+        return 3
+    tiles = [-(-w // tile_w) * -(-h // tile_h) for w, h in sizes]
+    slabs = n * len(tiles) // sum(tiles) >= 512 and 2 * max(tiles) <= 24576
+    longest = min(n, capacity)
+    return 6 + slabs + (longest > 4096) + (longest > 16384)
 
 
 # --------------------------------------------------------------------------- autotune
