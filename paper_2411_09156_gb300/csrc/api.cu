@@ -252,7 +252,6 @@ ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges
     const BinsLayout L = bins_layout(n, V, cap);
     if (cap > kMaxCapacity) return GES_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(bins, 0, 256, s) != cudaSuccess) return GES_ERR_CUDA;
     BinArgs a;
     a.n = n;
     a.n_views = n_views;
@@ -270,6 +269,7 @@ ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges
     a.aux = at<TileAux>(bins, L.aux);
     a.counts = at<uint32_t>(bins, L.counts);
     a.lists = at<uint4>(bins, L.lists);
+    a.stride = list_stride((uint64_t)L.n_tiles * depth_slabs(n, V), cap);
     a.jobs = at<uint4>(bins, L.jobs);
     a.places = at<uint32_t>(bins, L.places);
     a.cap = cap;

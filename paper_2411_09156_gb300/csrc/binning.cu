@@ -3,14 +3,14 @@
 //
 // Binning: the instances of every tile are counted, the counts scanned into segments, the instances
 // appended to their tile's segment in any order, and each segment sorted by (depth, entry) where it fits: in a
-// warp's, a part's or a whole CTA's shared memory. All counts stay in device memory, so the chain runs without
-// a host round trip and can be captured in a CUDA graph.
-// It replaced a depth sort of all entries (4 radix passes), the emission in that order and a stable
-// tile sort of all instances (2 or 3 passes), 28 launches that moved every instance about seven times.
-// Measured, the whole call as a graph, before and after: 1,000 splats at 128x128 88 -> 25 us; 100k at 800x800
-// 128 -> 55; 1.5M at 1600x1040 313 -> 280; 4 views of 300k 216 -> 160; 8 views of 1.5M (34.7M
-// instances) 1488 -> 1150. What bounds it there: the scattered 8-byte appends (425 us) and the sorts' shared-memory
-// traffic (430 us). Only lists far beyond a CTA got slower (1.5M splats in one 16x16 view: 224 -> 308 us).
+// warp's, a part's or a whole CTA's shared memory, after a split by depth where it does not. All counts stay in device
+// memory, so the chain runs without a host round trip and can be captured in a CUDA graph.
+// What bounds it: the scattered 8-byte appends and the sorts' shared-memory traffic (8 views of 1.5M splats of a
+// heightfield, 34.7M instances: 450 and 400 us of 1,140). The whole call as a graph against a depth sort of all entries
+// and a stable tile sort of all instances by radix passes: 1,000 splats at 128x128 26 us (95); 100k at 800x800 56 (131);
+// 1.5M at 1600x1040 280 (313); 4 views of 300k 161 (217); 8 of 1.5M 1,140 (1,490). Objects, whose tiles differ most
+// in length: 3 views of 170k 136 (157); 8 of 600k 490 (594). Slower where most instances lie in lists of thousands:
+// 1.5M splats of an object at 1600x1040 718 (574), in 8 views 2,271 (2,084).
 #include <cooperative_groups.h>
 
 #include "ges_internal.cuh"
@@ -299,7 +299,7 @@ __device__ __forceinline__ TileJob tile_job(const BinArgs &a, int v, size_t e, c
     return J;
 }
 
-// First kernel of a ges_bin: clears the counters and, if there are more instances than the capacity, finds where the
+// First kernel of a ges_bin: clears the header and the counters and, if there are more instances than the capacity, finds where the
 // lists end: the instances kept are the first `cap` of all in the order of (depth, entry, tile), so what is lost is the
 // farthest of every view. A radix selection over the entries' 64-bit keys (depth, entry), weighted by their tiles, by
 // the CTAs of one cluster, whose barrier and shared memory it needs; it leaves in the header the key of the entry
@@ -311,6 +311,7 @@ constexpr int kCutCtas = 8;
 __global__ void __cluster_dims__(kCutCtas, 1, 1) __launch_bounds__(1024) k_bin_begin(const BinArgs a, uint4 *clear,
                                                                                      uint64_t n_clear) {
     const uint32_t t = threadIdx.x, lane = t & 31u, rank = blockIdx.x;
+    if (rank == 0 && t < 64u) a.header[t] = 0u;  // (written further only by this CTA, past a barrier)
     for (uint64_t i = rank * 1024u + t; i < n_clear; i += kCutCtas * 1024u) clear[i] = make_uint4(0u, 0u, 0u, 0u);
     const unsigned long long total = *a.total;
     if (total <= a.cap || total >= 0xffffffffull) return;  // the same for the cluster
@@ -580,7 +581,14 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const BinArgs a, uint32_t pe
 // long for one CTA.
 __device__ __forceinline__ int seg_class(const BinArgs &a, uint32_t start, uint32_t n) {
     const uint32_t len = (uint32_t)(min((uint64_t)start + n, a.cap) - min((uint64_t)start, a.cap));
-    return len == 0u ? -1 : len <= 256u ? 0 : len <= 1024u ? 1 : len <= kCtaList ? 2 : len <= kBigList ? 3 : kListClasses;
+    return len == 0u ? -1 : len <= 256u ? 0 : len <= 1024u ? 1 : len <= kCtaList ? 2 : len <= kMidList ? 3
+         : len <= kBigList ? 4 : len <= kSplitList ? kToSplit : kListClasses;
+}
+
+// A list [s, e) of tile t to be sorted in chunks.
+__device__ __forceinline__ void push_chunks(const BinArgs &a, uint32_t s, uint32_t e, uint32_t t) {
+    const uint32_t nch = (e - s + kBigList - 1u) / kBigList, k = atomicAdd(&a.aux->n_jobs, nch);
+    for (uint32_t j = 0; j < nch; ++j) a.jobs[k + j] = make_uint4(s, e, t, j);
 }
 
 // Tile index, second part: each tile's range clipped to the capacity, its segments' starts (in place of their
@@ -673,11 +681,9 @@ __global__ void __launch_bounds__(1024) k_tile_index(const BinArgs a, uint32_t p
                 const uint32_t s = (uint32_t)min((uint64_t)at, a.cap), e = (uint32_t)min((uint64_t)end, a.cap);
                 if (cls >= 0 && cls < kListClasses) {
                     const uint32_t k = s_cls_base[cls] + atomicAdd(&s_cls[cls], 1u);
-                    a.lists[(size_t)cls * n_tiles * S + k] = make_uint4(s, e, t, 0u);
+                    a.lists[cls * a.stride + k] = make_uint4(s, e, t, 0u);
                 } else if (cls == kListClasses) {
-                    const uint32_t nch = (e - s + kBigList - 1u) / kBigList;
-                    const uint32_t k = atomicAdd(&a.aux->n_jobs, nch);
-                    for (uint32_t j = 0; j < nch; ++j) a.jobs[k + j] = make_uint4(s, e, t, j);
+                    push_chunks(a, s, e, t);
                 }
                 at = end;
             }
@@ -694,7 +700,8 @@ typedef unsigned long long u64;
 template <int ITEMS>
 __host__ __device__ constexpr int padded(int i) { return i + i / ITEMS; }
 
-// Merge sort of 64-bit keys by a group of threads, ITEMS consecutive keys a thread: a sorting network in
+// Merge sort of 64-bit keys by a group of threads (merges split along diagonals: Odeh, Green, Mwassi, Shmueli and Birk,
+// "Merge Path - parallel merging made simple", 2012), ITEMS consecutive keys a thread: a sorting network in
 // registers, then merges of doubling width, each thread producing its ITEMS outputs from where a binary
 // search along its diagonal says they start.
 // Sorts the len keys of sm (at padded<ITEMS>(i); len <= the group's threads x ITEMS) with the group's thread t; `sync`
@@ -844,15 +851,117 @@ __device__ __forceinline__ void sort_spread(int len, u64 *keys, uint32_t *cnt, u
 }
 
 // Sorts one segment (start, end, tile) of at most THREADS x ITEMS instances and writes its part of the lists.
-template <int THREADS, int ITEMS, class Sync>
+// SPLIT: split off a longer list, the keys (depth, entry) lie unsorted where the segment's own part of the lists will be.
+template <int THREADS, int ITEMS, bool SPLIT, class Sync>
 __device__ __forceinline__ void sort_segment(const BinArgs &a, uint4 rg, u64 *keys, uint32_t *cnt, uint32_t *scratch,
                                              int t, Sync &&sync) {
     sort_spread<THREADS, ITEMS>(
-        (int)(rg.y - rg.x), keys, cnt, scratch, t, sync, [&](int j) { return a.pairs[rg.x + j]; },
+        (int)(rg.y - rg.x), keys, cnt, scratch, t, sync,
+        [&](int j) {
+            return SPLIT ? ((u64)a.inst_tile[rg.x + j] << 32) | a.inst_entry[rg.x + j] : a.pairs[rg.x + j];
+        },
         [&](int at, u64 key) {
             a.inst_entry[rg.x + at] = (uint32_t)key;
             a.inst_tile[rg.x + at] = rg.z;
         });
+}
+
+// Splits the lists of kBigList to kSplitList entries by depth, a CTA each: a histogram over kSplitBins bins of equal
+// depth width, consecutive bins gathered into segments of about kSplitGroup entries, and the keys written bin by bin to
+// the list's own part of the outputs (depth and entry where tile and entry will be), from where the segments are sorted
+// like short lists. Bound by the scattered stores of the last of its three passes. Merged from chunks instead, whose
+// searches are one serial chain, the dense tiles of object scenes cost more than all else: 8 views of 1.5M splats (61M
+// instances) 800 us for 332 lists, 150 here; a 170k-splat batch of three 740x640 views 136 us for two, 33 here.
+constexpr int kSplitBins = 2048;
+__global__ void __launch_bounds__(1024) k_split_lists(const BinArgs a) {
+    __shared__ uint32_t s_bin[kSplitBins], s_warp[33], s_lo, s_hi, s_most;
+    __shared__ uint32_t s_start[kSplitList / kSplitGroup + 2], s_cls[2], s_base[2];
+    constexpr uint32_t kGroups = kSplitList / kSplitGroup + 1;
+    const uint32_t t = threadIdx.x, n = a.aux->n_list[kToSplit];
+    for (uint32_t k = blockIdx.x; k < n; k += gridDim.x) {
+        const uint4 rg = a.lists[kToSplit * a.stride + k];
+        const uint32_t len = rg.y - rg.x;
+        const uint32_t *high = reinterpret_cast<const uint32_t *>(a.pairs + rg.x) + 1;  // the depths
+        if (t == 0) { s_lo = 0xffffffffu; s_hi = 0u; s_most = 0u; }
+        if (t < 2u) s_cls[t] = 0u;
+        for (uint32_t b = t; b < kSplitBins; b += 1024u) s_bin[b] = 0u;
+        if (t <= kGroups) s_start[t] = 0xffffffffu;
+        __syncthreads();
+        // kRun loads in flight at a time: a list has few warps, and each pass waits for memory
+        constexpr uint32_t kRun = 8;
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (uint32_t j0 = t; j0 < len; j0 += kRun * 1024u) {
+#pragma unroll
+            for (uint32_t q = 0; q < kRun; ++q) {
+                const uint32_t z = high[2 * (size_t)min(j0 + q * 1024u, len - 1u)];
+                lo = min(lo, z);
+                hi = max(hi, z);
+            }
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((t & 31u) == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
+        __syncthreads();
+        const float z0 = __uint_as_float(s_lo), width = __uint_as_float(s_hi) - z0;
+        const float scale = width > 0.f ? (float)kSplitBins / width : 0.f;
+        auto bin = [&](uint32_t z) { return min((int)((__uint_as_float(z) - z0) * scale), kSplitBins - 1); };
+        for (uint32_t j0 = t; j0 < len; j0 += kRun * 1024u) {
+            uint32_t z[kRun];
+#pragma unroll
+            for (uint32_t q = 0; q < kRun; ++q) z[q] = high[2 * (size_t)min(j0 + q * 1024u, len - 1u)];
+#pragma unroll
+            for (uint32_t q = 0; q < kRun; ++q)
+                if (j0 + q * 1024u < len) atomicAdd(&s_bin[bin(z[q])], 1u);
+        }
+        __syncthreads();
+        // bin starts; a bin belongs to the segment its start falls into
+        const uint32_t c0 = s_bin[2 * t], c1 = s_bin[2 * t + 1];
+        uint32_t tot;
+        const uint32_t first = block_excl_scan(c0 + c1, s_warp, tot);
+        s_bin[2 * t] = first;
+        s_bin[2 * t + 1] = first + c0;
+        if (c0) atomicMin(&s_start[first / kSplitGroup], first);
+        if (c1) atomicMin(&s_start[(first + c0) / kSplitGroup], first + c0);
+        __syncthreads();
+        uint32_t at = 0, end = 0;
+        if (t < kGroups && s_start[t] != 0xffffffffu) {
+            at = s_start[t];
+            uint32_t g = t + 1u;
+            while (g < kGroups && s_start[g] == 0xffffffffu) ++g;
+            end = g < kGroups ? s_start[g] : len;
+            atomicMax(&s_most, end - at);
+        }
+        __syncthreads();
+        if (s_most > kCtaList) {  // the same for the CTA: left whole
+            if (t == 0) push_chunks(a, rg.x, rg.y, rg.z);
+        } else {
+            const int cls = end - at <= 1024u ? 0 : 1;
+            uint32_t place = 0;
+            if (end > at) place = atomicAdd(&s_cls[cls], 1u);
+            __syncthreads();
+            if (t < 2u) s_base[t] = s_cls[t] ? atomicAdd(&a.aux->n_list[kSplitShort + t], s_cls[t]) : 0u;
+            __syncthreads();
+            if (end > at)
+                a.lists[(kSplitShort + cls) * a.stride + s_base[cls] + place] = make_uint4(rg.x + at, rg.x + end, rg.z, 0u);
+            constexpr uint32_t kHalf = kRun / 2;
+            for (uint32_t j0 = t; j0 < len; j0 += kHalf * 1024u) {
+                u64 key[kHalf];
+#pragma unroll
+                for (uint32_t q = 0; q < kHalf; ++q) key[q] = a.pairs[rg.x + min(j0 + q * 1024u, len - 1u)];
+                uint32_t slot[kHalf];
+#pragma unroll
+                for (uint32_t q = 0; q < kHalf; ++q)
+                    if (j0 + q * 1024u < len) slot[q] = rg.x + atomicAdd(&s_bin[bin((uint32_t)(key[q] >> 32))], 1u);
+#pragma unroll
+                for (uint32_t q = 0; q < kHalf; ++q)
+                    if (j0 + q * 1024u < len) {
+                        a.inst_tile[slot[q]] = (uint32_t)(key[q] >> 32);
+                        a.inst_entry[slot[q]] = (uint32_t)key[q];
+                    }
+            }
+        }
+        __syncthreads();
+    }
 }
 
 // Lists of at most kCtaList entries: the longest by a whole CTA, those up to 1024 by 128 threads, those up to 256
@@ -863,16 +972,16 @@ __global__ void __launch_bounds__(kListThreads, 2) k_sort_lists(const BinArgs a)
     uint32_t *cnt = reinterpret_cast<uint32_t *>(sm + padded<kListItems>(kCtaList));
     __shared__ uint32_t scratch[3 * kListThreads / 32];
     const int t = threadIdx.x, g = t >> 7, w = t >> 5;
-    const size_t T = (size_t)a.V.n_tiles * a.slabs;
+    const size_t T = a.stride;
     const uint32_t n2 = a.aux->n_list[2], n1 = a.aux->n_list[1], n0 = a.aux->n_list[0];
     for (uint32_t k = blockIdx.x; k < n2; k += gridDim.x)
-        sort_segment<kListThreads, kListItems>(a, a.lists[2 * T + k], sm, cnt, scratch, t, []() { __syncthreads(); });
+        sort_segment<kListThreads, kListItems, false>(a, a.lists[2 * T + k], sm, cnt, scratch, t, []() { __syncthreads(); });
     for (uint32_t k = blockIdx.x * 4 + g; k < n1; k += gridDim.x * 4)
-        sort_segment<128, kListItems>(a, a.lists[T + k], sm + g * padded<kListItems>(1024), cnt + g * 1024, scratch + g * 12,
+        sort_segment<128, kListItems, false>(a, a.lists[T + k], sm + g * padded<kListItems>(1024), cnt + g * 1024, scratch + g * 12,
                                    t & 127, [&]() { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); });
     __syncthreads();
     for (uint32_t k = blockIdx.x * 16 + w; k < n0; k += gridDim.x * 16)
-        sort_segment<32, kListItems>(a, a.lists[k], sm + w * padded<kListItems>(256), cnt + w * 256, scratch, t & 31,
+        sort_segment<32, kListItems, false>(a, a.lists[k], sm + w * padded<kListItems>(256), cnt + w * 256, scratch, t & 31,
                                   []() { __syncwarp(); });
 }
 
@@ -884,23 +993,136 @@ __device__ __forceinline__ uint2 chunk_of(uint4 job, uint32_t q) {
 
 constexpr int kBigItems = (int)kBigList / 1024;
 
-// Lists of kCtaList to kBigList entries, and the chunks of longer ones (sorted in place).
+// sort_spread for up to kBigList keys by 1,024 threads, reading them three times (the range, the bucket counts, the
+// buckets) in place of holding 16 and their ranks a thread, which spilled. Bound by the shared-memory pipe. 1.5M splats
+// of an object at 1600x1040, 10.6M entries in lists of 4,096 to 11,323: k_sort_big 218 us with 16 keys a thread, 193
+// with this, 166 with this from 8,192 on and 8 keys a thread below. Stores come after every load.
+template <class Load, class Store>
+__device__ __forceinline__ void sort_spread_big(int len, u64 *keys, uint32_t *cnt, uint32_t *scratch, int t, Load &&load,
+                                                Store &&store) {
+    constexpr int WARPS = 32, kRun = 8;
+    const int lane = t & 31, w = t >> 5;
+    uint32_t zlo = 0xffffffffu, zhi = 0u;
+    for (int j0 = t; j0 < len; j0 += kRun * 1024) {
+#pragma unroll
+        for (int q = 0; q < kRun; ++q) {
+            const uint32_t z = (uint32_t)(load(min(j0 + q * 1024, len - 1)) >> 32);
+            zlo = min(zlo, z);
+            zhi = max(zhi, z);
+        }
+    }
+    int per = 1;  // buckets per thread
+    while (per * 1024 < len) per <<= 1;
+    const int nb = per * 1024;
+    for (int b = t; b < nb; b += 1024) cnt[b] = 0u;
+    zlo = __reduce_min_sync(0xffffffffu, zlo);
+    zhi = __reduce_max_sync(0xffffffffu, zhi);
+    if (lane == 0) { scratch[w] = zlo; scratch[WARPS + w] = zhi; }
+    __syncthreads();
+    zlo = __reduce_min_sync(0xffffffffu, scratch[lane]);
+    zhi = __reduce_max_sync(0xffffffffu, scratch[WARPS + lane]);
+    const float z0 = __uint_as_float(zlo), width = __uint_as_float(zhi) - z0;
+    const float scale = width > 0.f ? (float)nb / width : 0.f;
+    auto bucket = [&](u64 key) {
+        return min((int)((__uint_as_float((uint32_t)(key >> 32)) - z0) * scale), nb - 1);
+    };
+    for (int j0 = t; j0 < len; j0 += kRun * 1024) {
+        u64 k[kRun];
+#pragma unroll
+        for (int q = 0; q < kRun; ++q) k[q] = load(min(j0 + q * 1024, len - 1));
+#pragma unroll
+        for (int q = 0; q < kRun; ++q)
+            if (j0 + q * 1024 < len) atomicAdd(&cnt[bucket(k[q])], 1u);
+    }
+    __syncthreads();
+    uint32_t sum = 0, most = 0;
+    for (int q = 0; q < per; ++q) {
+        const uint32_t c = cnt[t * per + q];
+        sum += c;
+        most = max(most, c);
+    }
+    uint32_t incl = warp_incl_scan(sum);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 31) scratch[2 * WARPS + w] = incl;
+    if (lane == 0) scratch[w] = most;
+    __syncthreads();
+    most = __reduce_max_sync(0xffffffffu, scratch[lane]);
+    incl += __reduce_add_sync(0xffffffffu, lane < w ? scratch[2 * WARPS + lane] : 0u);
+    if (most <= kBucketMost) {  // the same in all threads
+        static_assert(kBigList <= 32767 && kBucketMost < 32, "a bucket's start, count and cursor in 15 + 5 + 5 bits");
+        uint32_t run = incl - sum;
+        for (int q = 0; q < per; ++q) {
+            const uint32_t c = cnt[t * per + q];
+            cnt[t * per + q] = run | (c << 15);
+            run += c;
+        }
+        __syncthreads();
+        for (int j0 = t; j0 < len; j0 += kRun * 1024) {
+            u64 k[kRun];
+#pragma unroll
+            for (int q = 0; q < kRun; ++q) k[q] = load(min(j0 + q * 1024, len - 1));
+#pragma unroll
+            for (int q = 0; q < kRun; ++q)
+                if (j0 + q * 1024 < len) {
+                    const uint32_t sc = atomicAdd(&cnt[bucket(k[q])], 1u << 20);
+                    keys[(sc & 0x7fffu) + (sc >> 20)] = k[q];
+                }
+        }
+        __syncthreads();
+        for (int j = t; j < len; j += 1024) {
+            const u64 key = keys[j];
+            const uint32_t sc = cnt[bucket(key)], first = sc & 0x7fffu, n = (sc >> 15) & 31u;
+            uint32_t at = first;
+            for (uint32_t q = 0; q < n; ++q) at += keys[first + q] < key;
+            store((int)at, key);
+        }
+    } else {
+        for (int j = t; j < len; j += 1024) keys[padded<kBigItems>(j)] = load(j);
+        __syncthreads();
+        sort_keys_apart<kBigItems>(keys, t, len, []() { __syncthreads(); });
+        for (int j = t; j < len; j += 1024) store(j, keys[padded<kBigItems>(j)]);
+    }
+    __syncthreads();
+}
+
+// Lists of kCtaList to kBigList entries, the segments split off longer ones (by 128 or 512 threads), and the chunks of
+// the longest (sorted in place). The CTAs take them in turn, the classes one after the other.
 __global__ void __launch_bounds__(1024) k_sort_big(const BinArgs a) {
     extern __shared__ u64 sm[];
     __shared__ uint32_t scratch[3 * 32];
     uint32_t *cnt = reinterpret_cast<uint32_t *>(sm + padded<kBigItems>(kBigList));
     const int t = threadIdx.x;
-    auto sync = []() { __syncthreads(); };
-    const uint32_t n3 = a.aux->n_list[3], nj = a.aux->n_jobs;
-    for (uint32_t k = blockIdx.x; k < n3; k += gridDim.x)
-        sort_segment<1024, kBigItems>(a, a.lists[3 * (size_t)a.V.n_tiles * a.slabs + k], sm, cnt, scratch, t, sync);
+    const uint32_t n3 = a.aux->n_list[3], n4 = a.aux->n_list[4], n6 = a.aux->n_list[kSplitShort],
+                   n7 = a.aux->n_list[kSplitLong], nj = a.aux->n_jobs;
+    const int g = t >> 7, h = t >> 9;
+    // this CTA's first of a class, after the `before` pieces of work of the classes before it
+    auto first = [](uint32_t before) { return (blockIdx.x + gridDim.x - before % gridDim.x) % gridDim.x; };
+    for (uint32_t k = first(0); k < n4; k += gridDim.x) {
+        const uint4 rg = a.lists[4 * a.stride + k];
+        sort_spread_big((int)(rg.y - rg.x), sm, cnt, scratch, t, [&](int j) { return a.pairs[rg.x + j]; },
+                        [&](int at, u64 key) {
+                            a.inst_entry[rg.x + at] = (uint32_t)key;
+                            a.inst_tile[rg.x + at] = rg.z;
+                        });
+    }
+    for (uint32_t k = first(n4); k < n3; k += gridDim.x)
+        sort_segment<1024, (int)kMidList / 1024, false>(a, a.lists[3 * a.stride + k], sm, cnt, scratch, t,
+                                                        []() { __syncthreads(); });
+    for (uint32_t k = first(n4 + n3) * 2 + h; k < n7; k += gridDim.x * 2)
+        sort_segment<512, 8, true>(a, a.lists[kSplitLong * a.stride + k], sm + h * padded<8>(4096), cnt + h * 4096,
+                                   scratch + h * 48, t & 511,
+                                   [&]() { asm volatile("bar.sync %0, 512;" ::"r"(h + 9) : "memory"); });
+    __syncthreads();
+    for (uint32_t k = first(n4 + n3 + (n7 + 1) / 2) * 8 + g; k < n6; k += gridDim.x * 8)
+        sort_segment<128, 8, true>(a, a.lists[kSplitShort * a.stride + k], sm + g * padded<8>(1024), cnt + g * 1024,
+                                   scratch + g * 12, t & 127,
+                                   [&]() { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); });
+    __syncthreads();
     for (uint32_t k = blockIdx.x; k < nj; k += gridDim.x) {
         const uint4 job = a.jobs[k];
         const uint2 c = chunk_of(job, job.w);
-        // (every key is in a register or in shared memory before the first is stored)
-        sort_spread<1024, kBigItems>((int)(c.y - c.x), sm, cnt, scratch, t, sync,
-                                     [&](int j) { return a.pairs[c.x + j]; },
-                                     [&](int at, u64 key) { a.pairs[c.x + at] = key; });
+        sort_spread_big((int)(c.y - c.x), sm, cnt, scratch, t, [&](int j) { return a.pairs[c.x + j]; },
+                        [&](int at, u64 key) { a.pairs[c.x + at] = key; });
     }
 }
 
@@ -1086,11 +1308,12 @@ cudaError_t launch_bin(const BinArgs &a, cudaStream_t s) {
     e = launch_instances<true>(c, shared, grid, threads, inst_smem, s);
     if (e != cudaSuccess) return e;
     // 4. sort: a tile's list has at most one entry per splat
+    const uint64_t longest = (uint64_t)a.n < a.cap ? (uint64_t)a.n : a.cap;
+    if (longest > kBigList) k_split_lists<<<2 * sms, 1024, 0, s>>>(a);
     constexpr int list_smem = (int)(sizeof(u64) * padded<kListItems>(kCtaList) + sizeof(uint32_t) * kCtaList);
     e = cudaFuncSetAttribute(k_sort_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, list_smem);
     if (e != cudaSuccess) return e;
-    k_sort_lists<<<(uint32_t)min((uint64_t)(2 * sms), (uint64_t)n_tiles * a.slabs), kListThreads, list_smem, s>>>(a);
-    const uint64_t longest = (uint64_t)a.n < a.cap ? (uint64_t)a.n : a.cap;
+    k_sort_lists<<<(uint32_t)min((uint64_t)(2 * sms), a.stride), kListThreads, list_smem, s>>>(a);
     if (longest > kCtaList) {
         constexpr int smem = (int)(sizeof(u64) * padded<kBigItems>(kBigList) + sizeof(uint32_t) * kBigList);
         e = cudaFuncSetAttribute(k_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

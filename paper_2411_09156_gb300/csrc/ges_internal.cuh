@@ -109,11 +109,15 @@ constexpr int kScanMaxPartials = 1024 * 16;
 
 inline uint32_t ceil_div_u64(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
-// Tile lists are sorted by CTAs: up to kCtaList entries by one CTA of 512 threads (or a part of one), up to
-// kBigList by one CTA of 1024, longer ones in chunks of at most kBigList.
-constexpr uint32_t kCtaList = 4096, kBigList = 16384;
+// Tile lists are sorted by CTAs: up to kCtaList entries by one CTA of 512 threads (or a part of one), up to kBigList by
+// one CTA of 1024, from registers up to kMidList. Longer ones, up to kSplitList, are first split by depth into segments of some kSplitGroup entries.
+// Where that leaves one beyond kCtaList (many equal depths, far outliers), and beyond kSplitList, a list is sorted in
+// chunks of at most kBigList that are merged.
+constexpr uint32_t kCtaList = 4096, kMidList = 8192, kBigList = 16384, kSplitList = 131072, kSplitGroup = 1024;
 constexpr int kLptBuckets = 128;   // list-length buckets of the longest-first queue
-constexpr int kListClasses = 4;    // <= 256, <= 1024, <= kCtaList, <= kBigList entries
+// lists of <= 256, <= 1024, <= kCtaList, <= kMidList, <= kBigList entries, those to split, segments split off of <= 1024
+// and of <= kCtaList
+constexpr int kListClasses = 8, kToSplit = 5, kSplitShort = 6, kSplitLong = 7;
 constexpr uint32_t kTileBlocks = 512;  // most CTAs of the tile-index kernels
 
 // Tiles per CTA of the tile-index kernels (a multiple of 1024), and their CTAs.
@@ -131,7 +135,7 @@ struct TileAux {
 
 // bins: [header 256][instance tile cap x 4][instance entry cap x 4][unsorted instances cap x 8][ranges T x 8]
 //       [queue T][tiles per length bucket of each tile-index CTA]
-//       [TileAux, counts of the G = T x slabs segments x 4][class lists 4 x G x 16][chunk jobs x 16]
+//       [TileAux, counts of the G = T x slabs segments x 4][class lists 8 x list_stride x 16][chunk jobs x 16]
 //       [places: CTAs per view x G x 4]
 // header: u32 n_inst (instances actually listed) at 0, u32 queue counters at 4 and 8, u64 count of
 // the forward's warp-cull passes at 16 (written only when the forward is asked for n_eval), the capacity's cut
@@ -192,6 +196,10 @@ inline bool inst_shared(int32_t n, const ViewSet &V) {
     return counters <= kSharedCounters && counters <= 16u * inst_entries(n, V.n_views);
 }
 
+// Entries of each sort class's list: the G segments, and what splitting the long ones adds (a segment of more than
+// kBigList entries gives at most one for each kSplitGroup of them and one more).
+inline uint64_t list_stride(uint64_t n_segs, uint64_t cap) { return n_segs + cap / (kSplitGroup / 2) + 1; }
+
 inline BinsLayout bins_layout(int32_t n, const ViewSet &V, uint64_t cap) {
     const uint32_t n_tiles = (uint32_t)V.n_tiles;
     const uint64_t n_segs = (uint64_t)n_tiles * depth_slabs(n, V);
@@ -205,7 +213,7 @@ inline BinsLayout bins_layout(int32_t n, const ViewSet &V, uint64_t cap) {
     L.queue = off; off = align256(off + (uint64_t)n_tiles * 4);
     L.buckets = off; off = align256(off + 4ull * kLptBuckets * tile_ctas(n_tiles));
     L.aux = off; L.counts = off + sizeof(TileAux); off = align256(L.counts + n_segs * 4);
-    L.lists = off; off = align256(off + n_segs * 16 * kListClasses);
+    L.lists = off; off = align256(off + list_stride(n_segs, cap) * 16 * kListClasses);
     // a list of more than kBigList entries has ceil(len / kBigList) < 2 len / kBigList chunks
     L.jobs = off; off = align256(off + (cap / (kBigList / 32) + 2) * 16);
     L.places = off;
@@ -487,7 +495,8 @@ struct BinArgs {
     uint32_t *buckets;  // [CTAs of the tile-index kernels][kLptBuckets]: tiles per length bucket
     TileAux *aux;
     uint32_t *counts;  // instances per segment (tile x slabs + slab), then the next free slot of it
-    uint4 *lists;      // [kListClasses][segments]: start, end, tile, -
+    uint4 *lists;      // [kListClasses][stride]: start, end, tile, -
+    uint64_t stride;
     uint4 *jobs;       // start, end, tile, chunk
     uint32_t *places;  // [CTAs of the instance kernels per view][segments]: where a CTA's instances of one start
     uint32_t slabs;
