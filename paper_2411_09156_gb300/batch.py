@@ -201,11 +201,11 @@ def binning_launches(n: int, sizes, tile_w: int, tile_h: int, capacity: int) -> 
     """Kernels one ges_bin launches for n splats in views of these sizes: the counters and two index launches;
     with splats, the tile counts, the appends and the sort of ordinary lists too, a depth-range pass where
     tiles are split by depth (512 entries or more a tile, and twice the largest view's tiles within the
-    24,576 counters of a CTA's shared memory), and what a list of up to min(n, capacity) may need."""
+    22,528 counters of a CTA's shared memory), and what a list of up to min(n, capacity) may need."""
     if n == 0:
         return 3
     tiles = [-(-w // tile_w) * -(-h // tile_h) for w, h in sizes]
-    slabs = n * len(tiles) // sum(tiles) >= 512 and 2 * max(tiles) <= 24576
+    slabs = n * len(tiles) // sum(tiles) >= 512 and 2 * max(tiles) <= 22528
     longest = min(n, capacity)
     return 6 + slabs + (longest > 4096) + 2 * (longest > 16384)
 

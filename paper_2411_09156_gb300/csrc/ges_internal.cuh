@@ -148,7 +148,9 @@ struct BinsLayout {
 
 // The instance kernels: CTAs of up to kInstThreads, each with consecutive entries of one view.
 constexpr int kInstThreads = 512;
-constexpr uint32_t kSharedCounters = 24576;  // most counters in shared memory (96 KB: two CTAs per SM)
+// Most counters in shared memory: with the 24 KB of jobs beside them two CTAs still fit an SM (24,000 counters, one CTA:
+// 1.5M splats in a 1600x960 view, 8x8 tiles, 595 us against 407 with the counters in global memory).
+constexpr uint32_t kSharedCounters = 22528;
 constexpr uint32_t kMostSlabs = 64;
 
 // Entries per CTA: more share a tile's atomic and write its instances side by side, up to 8 rounds of
@@ -190,10 +192,15 @@ inline uint32_t depth_slabs(int32_t n, const ViewSet &V) {
 }
 
 // Whether a CTA counts its entries' instances in shared memory: its counters are cleared and read once a CTA, which
-// its entries have to pay for.
+// its entries have to pay for. Shared and global by counters per entry of a CTA (one 1600x1040 view in 16x8 tiles,
+// heightfield and object): 68 an entry 115, 155 and 83, 115 us; 37 107, 161 and 95, 173; 25 107, 193 and 103, 208;
+// 13 171, 375 and 189, 406; 6 291, 770 and 364, 819. Above 18,432 counters, where two CTAs are all that fit, half as many:
+// 8x8 tiles, 1.5M splats, 22,500 counters: one view (11 an entry) 436, 1,078 and 362, 968; four (5.5) 933, 2,036 and
+// 1,282, 2,260.
 inline bool inst_shared(int32_t n, const ViewSet &V) {
     const uint32_t counters = most_tiles(V) * depth_slabs(n, V);
-    return counters <= kSharedCounters && counters <= 16u * inst_entries(n, V.n_views);
+    const uint32_t each = counters <= 18432u ? 16u : 8u;
+    return counters <= kSharedCounters && counters <= each * inst_entries(n, V.n_views);
 }
 
 // Entries of each sort class's list: the G segments, and what splitting the long ones adds (a segment of more than

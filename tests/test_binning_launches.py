@@ -16,8 +16,8 @@ from paper_2411_09156_gb300.batch import binning_launches
     (512 * 2500, [(800, 800), (800, 801)], (16, 16), 1 << 24, 9),
     # as dense, but two counters for each of 13,000 tiles do not fit: no split by depth, no depth-range pass
     (7_000_000, [(1600, 1040)], (16, 8), 1 << 26, 9),
-    # 12,288 tiles do
-    (7_000_000, [(2048, 768)], (16, 8), 1 << 26, 10),
+    # 11,264 tiles do
+    (7_000_000, [(2048, 704)], (16, 8), 1 << 26, 10),
 ])
 def test_launch_count(n, sizes, tile, capacity, launches):
     assert binning_launches(n, sizes, *tile, capacity) == launches
