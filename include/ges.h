@@ -350,7 +350,7 @@ GES_API ges_status ges_knn(int32_t n, const float *pos_op, void *workspace, size
  * along a level-set ray (Sec. 3.3, "Mesh Extraction": the start point's 16 closest
  * splats, as in Sec. 4.2); ges_levelset calls the same search.
  *   points   [m, 4] float32 (x, y, z, w), 16-byte aligned; w = 0 marks a point without a
- *            query (its list is all -1)
+ *            query (its list is all -1, as that of a point with a NaN coordinate is)
  *   knn      [m, 16] int32 (written, 16-byte aligned): point j's neighbours by increasing
  *            distance, ties to the lower index
  * The points are searched in grid-cell order; cells are grouped in 4 x 4 x 4 blocks whose

@@ -115,7 +115,8 @@ __device__ __forceinline__ void red_add4(float *p, float x, float y, float z, fl
 // of one neighbour slot together, consecutive lanes taking consecutive 16-byte pieces, two slots ahead,
 // past L1 (a splat's neighbours are scattered: through L1 the copies of 20 warps evict one another, 1.76 ms).
 // Forward and backward at 1.5M samples, the whole call: 1.41 ms with scalar reductions and own loads,
-// 1.20 with vector reductions, 0.94 with staged records (two stages: 0.98; 7 CTAs per SM: 1.06).
+// 1.20 with vector reductions, 0.94 with staged records (two stages: 0.98; 7 CTAs per SM: 1.06), 0.90 with the
+// accumulators cleared by a memory set and the sums added by 1,024 threads.
 constexpr int kStages = 3;
 struct GsrStage {
     int nb[32][GES_KNN_K + 1];       // the lanes' neighbour lists (padded: a column's entries in distinct banks)

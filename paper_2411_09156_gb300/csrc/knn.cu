@@ -9,12 +9,12 @@
 // distances alone, then, over the cells within the 16th, for the centres themselves. Rows of
 // cells farther than the current 16th are skipped and the others cut to it along x, which keeps
 // queries away from the centres (points in front of a surface) from reading every cell of their
-// block. (Cells, whole call: 2 per point, 1, 1/2: KNN of a 1.5M-splat heightfield 1.24, 1.26, 1.50 ms, of
-// a 300k-splat object 1.52, 1.02, 0.92; level-set points of a 1600x1040 view 3.00, 2.58, 2.48.) Queries run in
-// cell order, so a warp searches one neighbourhood. Distances are squared float32 with a fixed operation order; ties go to
+// block. One cell per point: with two and with a half KNN of a 1.5M-splat heightfield takes 1.24 and 1.50 ms
+// against 1.26, of a 300k-splat object 1.52 and 0.92 against 1.02. Queries run in cell order, so a warp searches
+// one neighbourhood. Distances are squared float32 with a fixed operation order; ties go to
 // the lower index. A query that would examine more than 131,072 candidates (a bound that well-spread
-// centres never reach; tens of thousands of coincident centres would) takes the best of the first
-// 131,072 in ring order instead, so no input makes the search quadratic.
+// centres never reach; more coincident centres than that would) takes the best of the first 131,072 in ring
+// order instead, and one that no distance bounds ends at once, so no input makes the search quadratic.
 #include "ges_internal.cuh"
 #include "sort_net.cuh"
 
@@ -30,7 +30,8 @@ constexpr uint32_t kQueryBudget = 1u << 17;  // candidate points one query may e
 // 7.3 in one pass (before the two passes: 6.6); 100,000: 75.7, 27.9, 15.1 (9.0 with half the budget). Ordinary queries
 // examine a few hundred.
 constexpr uint32_t kTwoPassMost = 2048;
-// 16 CTAs of 64 threads per SM (64 registers): at 12 or 20 the centre queries take 11 % or 1 % longer
+// 16 CTAs of 64 threads per SM (64 registers): at 12 or 20 the centre queries take 11 % or 1 % longer, as 32 one-warp CTAs
+// the whole call of either query 1 %
 constexpr int kQueryThreads = 64, kQueryCtas = 16;
 // The first pass ends when the searched cells reach sqrt(kReach) of the 16th distance: the second pass then
 // drops the few candidates too many, which costs less than another ring (reach 1: 1.61 ms against 1.42-1.45
@@ -894,8 +895,6 @@ cudaError_t knn_points_run(int32_t n, const float4 *pos, int32_t m, const float4
                    at<uint32_t>(qws, Q.partials), s);
     if (e != cudaSuccess) return e;
     const int res = ((Q.bits + 7) / 8) & 1;
-    // one warp per CTA: query walks differ widely in length, and a CTA of several warps would hold
-    // its slot until its longest walk ended
     k_knn_points<<<ceil_div_u64(m, kQueryThreads), kQueryThreads, 0, s>>>(at<float4>(workspace, L.spos), at<uint32_t>(workspace, L.starts),
                                                      at<uint32_t>(workspace, L.bcount), at<KnnGrid>(workspace, L.grid),
                                                      pts, vals[res], m, knn);

@@ -190,8 +190,8 @@ __device__ __forceinline__ bool load_cull_stage(const float4 *rec, uint32_t e, u
 // its own list (the loop runs for the longer list): 13 % fewer warp instructions on the 300k-splat
 // 8-view batch, 1.68 -> 1.58 ms on the 1.5M-splat one. Four 4x2 groups (a cull test and a shared-memory
 // address each) took 1.85 ms. The packed operations bring the staged pairs into registers as they are
-// used, and with the cap of 36 warps per SM (56 registers; 40 warps spill: 1.71 ms) the kernel takes
-// 1.54 ms (train, one 1600x1040 view: 0.409 -> 0.379). Every value is rounded as before, bit for bit.
+// used, and with the cap of 36 warps per SM (56 registers; with depth and normal 12 bytes spill, at 40 warps so
+// much that it takes 1.71 ms) the kernel takes 1.54 ms (train, one 1600x1040 view: 0.409 -> 0.379). Every value is rounded as before, bit for bit.
 // DN: the depth and normal outputs are wanted; without them (the training step renders for a
 // loss on the colour) their accumulations drop out.
 template <int TW, int TH, bool DN>
