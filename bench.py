@@ -238,14 +238,14 @@ def hbm_stage_fractions(plan, sc, cams, n_inst: int, flush, hbm: float, warmup: 
     """Preprocess (K1), binning (K2-K5) and preprocess backward (K8) timed alone (eager calls,
     L2 flushed) against the measured HBM copy bandwidth, with the algorithmic bytes per unit of
     the method: K1 reads each splat's attributes once (48 B + the colour) and writes a 64 B render
-    and a 32 B binning record per (splat, view); binning moves 28 B per (splat, view) and 44 B per
-    instance; K8 reads the 64 B screen gradient per (splat, view) and each splat's attributes and
+    and a 32 B binning record per (splat, view); binning reads that record twice and moves 24 B per
+    instance (its key written and read, its tile and entry written); K8 reads the 64 B screen gradient per (splat, view) and each splat's attributes and
     writes its gradients once."""
     r, x = plan.rast, plan.inputs
     n, nv = sc.n, sc.n * len(cams)
     col = x[3].numel() * x[3].element_size() // max(n, 1)
     b_k1 = n * (48 + col) + nv * 96
-    b_bin = 28 * nv + 44 * n_inst
+    b_bin = 64 * nv + 24 * n_inst
     b_k8 = nv * 64 + n * (48 + col) + n * (48 + 4 * (col // x[3].element_size()))
     t_k1 = timed_call(lambda: r.preprocess(*x), warmup, steps, flush, world)
     t_bin = timed_call(lambda: r.bin(), warmup, steps, flush, world)
