@@ -274,6 +274,7 @@ ges_status ges_bin(int32_t n, int32_t n_views, const ges_camera *cams, const ges
     a.places = at<uint32_t>(bins, L.places);
     a.cap = cap;
     a.per_cta = a.parts = 0;
+    a.own = false;
     a.slabs = depth_slabs(n, V);
     a.build_queue = cfg->persistent != 0;
     a.V = V;

@@ -6,11 +6,12 @@
 // warp's, a part's or a whole CTA's shared memory, after a split by depth where it does not. All counts stay in device
 // memory, so the chain runs without a host round trip and can be captured in a CUDA graph.
 // What bounds it: the scattered 8-byte appends and the sorts' shared-memory traffic (8 views of 1.5M splats of a
-// heightfield, 34.7M instances: 450 and 400 us of 1,140). The whole call as a graph against a depth sort of all entries
+// heightfield, 34.7M instances: 410 and 400 us of 1,035). The whole call as a graph against a depth sort of all entries
 // and a stable tile sort of all instances by radix passes: 1,000 splats at 128x128 26 us (95); 100k at 800x800 56 (131);
-// 1.5M at 1600x1040 280 (313); 4 views of 300k 161 (217); 8 of 1.5M 1,140 (1,490). Objects, whose tiles differ most
-// in length: 3 views of 170k 136 (157); 8 of 600k 490 (594). Slower where most instances lie in lists of thousands:
-// 1.5M splats of an object at 1600x1040 718 (574), in 8 views 2,271 (2,084).
+// 1.5M at 1600x1040 271 (313); 4 views of 300k 163 (217); 8 of 1.5M 1,035 (1,490). Objects, whose tiles differ most
+// in length: 3 views of 170k 136 (157); 8 of 600k 454 (594). Slower where most instances lie in lists of thousands, and
+// one view's segments outgrow L2: 2M splats of an object at 1600x1040 595 (517) in 16x16 tiles, 1,012 (732) in 16x8;
+// 8 views of 1.5M 2,127 (2,084).
 #include <cooperative_groups.h>
 
 #include "ges_internal.cuh"
@@ -384,6 +385,54 @@ __global__ void __cluster_dims__(kCutCtas, 1, 1) __launch_bounds__(1024) k_bin_b
                      });
 }
 
+// The instances of entries whose box has more than 32 tiles: the tile tests again.
+template <class OnInstance>
+__device__ __forceinline__ void large_box_instances(const BinArgs &a, int v, bool big, const uint4 b0, size_t e, uint4 *jobs,
+                                                    int lane, uint32_t part, OnInstance &&on_instance) {
+    if (!__any_sync(0xffffffffu, big)) return;
+    const int tiles_x = a.V.tiles_x[v];
+    const uint32_t tbase = (uint32_t)a.V.tile_base[v];
+    const int tw = a.V.tile_w, th = a.V.tile_h;
+    const int lw = __ffs(tw) - 1, lh = __ffs(th) - 1;  // tile sides are powers of two
+    TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
+    if (big) J = tile_job(a, v, e, b0, lw, lh);
+    warp_tile_rounds(J, lane, lw, lh, tw, th, jobs, part, a.parts,
+                     [&](uint32_t, uint32_t, uint32_t, uint32_t, int tx, int ty, uint32_t owner, bool hit) {
+                         const uint32_t depth = __shfl_sync(0xffffffffu, b0.w, owner);
+                         const uint32_t ent = __shfl_sync(0xffffffffu, (uint32_t)e, owner);
+                         if (hit) on_instance(tbase + (uint32_t)(ty * tiles_x + tx), depth, ent);
+                     });
+}
+
+// The instances of a lane's own entry from its hit mask, four at a time: take(tile, depth) for each, then put(what it
+// returned, depth, entry), so that four of take's atomics are in flight. It issues a third of the instructions that sharing
+// them over the warp does (8 views of 1.5M splats of a heightfield: count 262 -> 204 us, of an object 417 -> 330), and is
+// used where the atomics are in shared memory: waiting for global ones, few lanes in flight, a 200k-splat object in a
+// 1600x1040 view took 164 us against 124.
+template <class Take, class Put>
+__device__ __forceinline__ void lane_instances(const BinArgs &a, int v, uint32_t depth, const uint4 b1, uint32_t e, Take &&take,
+                                               Put &&put) {
+    constexpr uint32_t kNone = 0xffffffffu;
+    const uint32_t tiles_x = (uint32_t)a.V.tiles_x[v], rw = b1.z & 0xffffu;
+    const uint32_t origin = (uint32_t)a.V.tile_base[v] + (b1.y >> 16) * tiles_x + (b1.y & 0xffffu);
+    const uint32_t mdiv = (65536u + rw - 1u) / rw, down = tiles_x - rw;  // bit / rw == (bit * mdiv) >> 16 for bit < 32
+    for (uint32_t m = b1.x; m;) {
+        uint32_t slot[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            slot[q] = kNone;
+            if (m) {
+                const uint32_t bit = (uint32_t)__ffs(m) - 1u;
+                m &= m - 1u;
+                slot[q] = take(origin + bit + ((bit * mdiv) >> 16) * down, depth);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (slot[q] != kNone) put(slot[q], depth, e);
+    }
+}
+
 // The instances of a warp's 32 entries, each listed tile of each entry once: on_instance(global tile, depth bits,
 // entry) is called by one lane each. Entries whose box has at most 32 tiles are expanded from their hit masks
 // by the whole warp, 32 instances a round (instance j goes to the entry whose prefix interval holds j, binary
@@ -424,22 +473,10 @@ __device__ __forceinline__ void warp_instances(const BinArgs &a, int v, uint32_t
                         (uint32_t)e - (uint32_t)lane + (uint32_t)owner);
         }
     }
-    const bool big = tiles && !rw;
-    if (!__any_sync(0xffffffffu, big)) return;
-    const int tw = a.V.tile_w, th = a.V.tile_h;
-    const int lw = __ffs(tw) - 1, lh = __ffs(th) - 1;  // tile sides are powers of two
-    TileJob J = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, 0u};
-    if (big) J = tile_job(a, v, e, b0, lw, lh);
-    warp_tile_rounds(J, lane, lw, lh, tw, th, jobs, part, a.parts,
-                     [&](uint32_t, uint32_t, uint32_t, uint32_t, int tx, int ty, uint32_t owner, bool hit) {
-                         const uint32_t depth = __shfl_sync(0xffffffffu, b0.w, owner);
-                         const uint32_t ent = __shfl_sync(0xffffffffu, (uint32_t)e, owner);
-                         if (hit) on_instance(tbase + (uint32_t)(ty * tiles_x + tx), depth, ent);
-                     });
+    large_box_instances(a, v, tiles && !rw, b0, e, jobs, lane, part, on_instance);
 }
-
 // EMIT false: counts the instances per tile. EMIT true: appends each instance to its tile's segment.
-// A CTA takes `a.per_cta` entries of one view, the views in turn. SHARED: it counts them per tile in shared memory
+// A CTA takes `a.per_cta` entries of one view. SHARED: it counts them per tile in shared memory
 // first, so that a tile costs one global atomic per CTA: the atomics of all CTAs on a view's few counters were
 // what the kernel waited for (8 views of 1.5M splats, 34.7M instances: count 0.91 and append 1.06 ms with an
 // atomic per instance). The count keeps what those atomics return, the CTA's place among a tile's instances, and
@@ -455,10 +492,14 @@ __global__ void __launch_bounds__(kInstThreads, EMIT || SLABS ? 3 : 4) k_instanc
     extern __shared__ uint32_t s_cnt[];  // SHARED: instances per segment of the view; the CTA's next slot in each
     __shared__ uint4 s_jobs[kInstThreads / 32][kJobWords * 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // The append takes the views one after the other: the segments it has open then are one view's and mostly stay in L2
+    // until their sectors are full (8 views of 1.5M splats: 453 -> 411 us against all views at once). The count takes them
+    // in turn, which keeps its atomics from meeting on one small view's counters.
     // blocks: the views of a part of a run of entries, the parts (every a.parts-th round of 32 instances of a
     // warp's entries: few splats of many tiles each give too few warps otherwise), the runs
-    const int v = (int)(blockIdx.x % (uint32_t)a.n_views);
-    const uint32_t row = blockIdx.x / (uint32_t)a.n_views, part = row % a.parts;
+    const uint32_t nv = (uint32_t)a.n_views, rows = gridDim.x / nv;
+    const int v = (int)(EMIT && SHARED ? blockIdx.x / rows : blockIdx.x % nv);
+    const uint32_t row = EMIT && SHARED ? blockIdx.x % rows : blockIdx.x / nv, part = row % a.parts;
     const uint32_t i0 = row / a.parts * a.per_cta, i1 = min(i0 + a.per_cta, (uint32_t)a.n);
     const uint32_t S = SLABS ? a.slabs : 1u, tbase = (uint32_t)a.V.tile_base[v] * S, vtiles = (uint32_t)a.V.tile_base[v + 1] * S - tbase;
     float z0 = 0.f, per_z = 0.f;
@@ -498,6 +539,24 @@ __global__ void __launch_bounds__(kInstThreads, EMIT || SLABS ? 3 : 4) k_instanc
             if (key < last || (key == last && tile < a.header[kCutWord + 2])) on_instance(tile, depth, e);
         });
     };
+    // each entry's instances by its own lane (no cut applies, and a warp has its entries to itself)
+    auto each_own = [&](auto &&take, auto &&put) {
+        for (uint32_t w0 = i0 + (uint32_t)warp * 32u; w0 < i1; w0 += blockDim.x) {
+            const uint32_t i = w0 + (uint32_t)lane;
+            const size_t e = (size_t)v * a.n + i;
+            uint4 b0 = make_uint4(0u, 0u, 0u, 0u), b1 = b0;
+            if (i < i1) {
+                b0 = __ldg(a.binrec + 2 * e);
+                b1 = __ldg(a.binrec + 2 * e + 1);
+            }
+            const bool masked = (b1.z & 0xffffu) * (b1.z >> 16) <= 32u;
+            if (b0.z && masked) lane_instances(a, v, b0.w, b1, (uint32_t)e, take, put);
+            __syncwarp();
+            large_box_instances(a, v, b0.z && !masked, b0, e, s_jobs[warp], lane, 0u,
+                                [&](uint32_t tile, uint32_t depth, uint32_t ent) { put(take(tile, depth), depth, ent); });
+        }
+    };
+    const bool own = !cut && a.own;
     auto append = [&](uint32_t slot, uint32_t depth, uint32_t e) {
         if (slot < a.cap) a.pairs[slot] = ((unsigned long long)depth << 32) | e;
         else set_error(a.err, kErrCapacity);  // (counts beyond the total only: the cut keeps within the capacity)
@@ -508,12 +567,20 @@ __global__ void __launch_bounds__(kInstThreads, EMIT || SLABS ? 3 : 4) k_instanc
         for (uint32_t t = threadIdx.x; t < vtiles; t += blockDim.x) s_cnt[t] = EMIT ? a.counts[tbase + t] + place[t] : 0u;
         __syncthreads();
         if (EMIT) {
-            each([&](uint32_t tile, uint32_t depth, uint32_t e) {
-                append(atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u), depth, e);
-            });
+            if (own)
+                each_own([&](uint32_t tile, uint32_t depth) { return atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u); },
+                         append);
+            else
+                each([&](uint32_t tile, uint32_t depth, uint32_t e) {
+                    append(atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u), depth, e);
+                });
             return;
         }
-        each([&](uint32_t tile, uint32_t depth, uint32_t) { atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u); });
+        if (own)
+            each_own([&](uint32_t tile, uint32_t depth) { atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u); return 0u; },
+                     [](uint32_t, uint32_t, uint32_t) {});
+        else
+            each([&](uint32_t tile, uint32_t depth, uint32_t) { atomicAdd(&s_cnt[segment(tile, depth) - tbase], 1u); });
         __syncthreads();
         for (uint32_t t = threadIdx.x; t < vtiles; t += blockDim.x) {
             const uint32_t c = s_cnt[t];
@@ -1291,6 +1358,7 @@ cudaError_t launch_bin(const BinArgs &a, cudaStream_t s) {
     const bool shared = inst_shared(a.n, a.V);  // as the layout was made for
     c.per_cta = inst_entries(a.n, a.n_views);
     c.parts = inst_parts(a.n, a.n_views);
+    c.own = c.parts == 1u;
     const uint32_t grid = ceil_div_u64((uint64_t)a.n, c.per_cta) * c.parts * (uint32_t)a.n_views;
     const uint32_t threads = min(c.per_cta, (uint32_t)kInstThreads);
     const int inst_smem = shared ? (int)(sizeof(uint32_t) * counters) : 0;

@@ -509,6 +509,7 @@ struct BinArgs {
     uint32_t slabs;
     uint64_t cap;
     uint32_t per_cta, parts;  // entries a CTA of the instance kernels takes, CTAs that share them
+    bool own;                 // each entry's instances by its own lane
     bool build_queue;
     ViewSet V;
 };
